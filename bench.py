@@ -121,7 +121,8 @@ def kernel_sha(files=NCU_TRAFFIC[("gktl", "step_kernel<fp32, vec=4>")]["files"])
 
 def kernel_label(L, variant: int, storage: str) -> str:
     _, vec, warps = L.lbm_step_variant_info(variant)
-    name = "step_rows_kernel" if L.lbm_step_variant_kind(variant) == 1 else "step_kernel"
+    name = {1: "step_rows_kernel", 2: "step_tb_kernel", 3: "step_stream_kernel"}.get(
+        L.lbm_step_variant_kind(variant), "step_kernel")
     return f"{name}<{storage}, vec={vec}, warps={warps}>"
 
 
@@ -469,6 +470,8 @@ def run_ours(args):
     hbm, peak_kind = peaks()
     avg_launch_ms = st_ms / max(st_launches, 1)
     bytes_per_site = BYTES_PER_SITE if args.storage == "fp32" else BYTES_PER_SITE // 2
+    if L.lbm_step_variant_kind(variant) == 3:  # two steps per pass over the populations
+        bytes_per_site //= 2
     achieved = bytes_per_site * sites / (avg_launch_ms / 1e3) / 1e9
     traffic = None
     rec = NCU_TRAFFIC.get((args.workload, traffic_key(label)))

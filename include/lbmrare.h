@@ -281,13 +281,18 @@ int lbm_ensemble_autotune(lbm_ensemble* e, int32_t* variant);
  * describe any index.  Without a forced variant, step calls over at most 2^18
  * sites (clones x nx x ny, e.g. one AMS branch) use a separate small-list
  * variant (default: the narrowest register-staged variant with 8 warps, which
- * puts the most threads on a small grid); lbm_ensemble_autotune picks both. */
+ * puts the most threads on a small grid); lbm_ensemble_autotune picks both.
+ * Step calls of four steps and more over many rows of periodic channels stream
+ * rows, two steps per pass over memory, unless a variant is forced; the
+ * populations and the drag are the default variant's bit for bit. */
 int lbm_ensemble_set_variant(lbm_ensemble* e, int32_t variant);
 int lbm_step_variant_info(int32_t variant, int32_t* storage, int32_t* vec, int32_t* warps);
 int32_t lbm_step_variant_count(void);
 /* Data movement of a variant: 0 = register-staged row segments, one warp per
  * segment (lbm_step.cuh); 1 = whole rows staged in shared memory by bulk
- * copies (lbm_step_rows.cuh).  LBM_ERR_ARG for an index out of range. */
+ * copies (lbm_step_rows.cuh); 2 = tiles in shared memory, up to three steps per
+ * launch (lbm_step_tb.cuh); 3 = rows streamed through a block, two steps per
+ * pass over memory (lbm_step_stream.cuh).  LBM_ERR_ARG for an index out of range. */
 int32_t lbm_step_variant_kind(int32_t variant);
 
 /* Failure-detection self test of the bounded device-side waits used by the

@@ -31,11 +31,12 @@ struct StepVariant {
     cudaError_t (*launch)(const StepParams&, cudaStream_t);
     int kind;   // 0: register-staged row segments per warp; 1: whole rows staged by bulk copies;
                 // 2: tiles in shared memory, several steps per launch (temporal blocking)
+                // 3: rows streamed through a block, two steps per launch
     bool (*supports)(const StepParams&);  // null: every shape
     // the open channel's step (fused step + boundary columns); null: this
     // variant has no open-channel instantiation
     Launch launch_open = nullptr;
-    int multi = 1;  // most steps one launch runs (kind 2; an odd number per launch)
+    int multi = 1;  // most steps one launch runs (kind 2: an odd number per launch; kind 3: one or two)
 };
 
 // LBM_ERR_ARG unless the collision fields of c are valid (lbm_ensemble.cu)
@@ -127,6 +128,8 @@ struct lbm_ensemble {
     // calls over many sites, one for calls below kSmallSites (an AMS branch)
     int variant;
     int variant_small;
+    bool variant_forced;      // by lbm_ensemble_set_variant: runs every call
+    bool variant_tuned;       // by lbm_ensemble_autotune
     // step chunks captured once as CUDA graphs and replayed: one cached
     // executable per (variant, clone list, list length, chunk length)
     struct StepGraph {

@@ -464,7 +464,7 @@ Ring ring_for(const lbm_config& c, int vec, int kind)
         r.n_slots = (r.ry1 / kTbTy - r.ry0 / kTbTy + 1) * (r.rs1 - r.rs0 + 1);
         return r;
     }
-    if (kind == 0) {
+    if (kind == 0 || kind == 3) {
         const int seg_w = 32 * vec;
         r.rs0 = (c.obs_x0 - 1) / seg_w;
         r.rs1 = (c.obs_x0 + c.obs_w) / seg_w;
@@ -500,11 +500,6 @@ int default_variant_small(int storage, bool open)
         if (v[i].storage == storage && v[i].kind == 0 && v[i].warps == 8 && (best < 0 || v[i].vec < v[best].vec))
             best = (int)i;
     return best >= 0 ? best : default_variant(storage);
-}
-
-int variant_for(const lbm_ensemble* e, int n_list)
-{
-    return (int64_t)n_list * e->cfg.nx * e->cfg.ny <= kSmallSites ? e->variant_small : e->variant;
 }
 
 // parameters of step `step` (0-based) of a chunk of `chunk` steps (chunk 0: a
@@ -549,6 +544,7 @@ StepParams make_params(const lbm_ensemble* e, const int32_t* list, int32_t n_lis
     p.scale = e->scale;
     p.inv_scale = e->inv_scale;
     p.step_in_batch = step;
+    p.flip = step & 1;
     p.tb_steps = 1;
     const Solids sol = solids_of(c);
     p.open = c.open_x;
@@ -578,6 +574,41 @@ StepParams make_params(const lbm_ensemble* e, const int32_t* list, int32_t n_lis
         p.bc_pre = (float)(-2.0 / 3.0 * (open_tau(c, c.nx - 1) - 1.0));
     }
     return p;
+}
+
+// the row-streaming variant of a storage format (-1: none)
+int stream_variant(int storage)
+{
+    const auto& v = step_variants();
+    for (size_t i = 0; i < v.size(); ++i)
+        if (v[i].storage == storage && v[i].kind == 3) return (int)i;
+    return -1;
+}
+
+// the variant of a step call over n_list clones.  A call of four steps and more
+// on a periodic channel streams rows, two steps per pass over memory, if every
+// block then has enough rows: a block recomputes two rows of its span, and each
+// of its rows waits on the one before.  Measured on channels of 128 to 2048
+// columns (single steps / streamed, us per step): FP32 BGK 16.6 / 17.1 at 5
+// rows a block, 23.1 / 19.9 at 7, 37.0 / 26.1 at 10, 178 / 105 at 54; FP32
+// central moments 24.6 / 26.0 at 7, 36.9 / 33.3 at 10; FP16 BGK 14.9 / 15.6 at
+// 7, 24.2 / 20.3 at 10; FP16 central moments 30.2 / 30.7 at 10, 39.2 / 36.8 at 13.
+int variant_for(const lbm_ensemble* e, int n_list, int n_steps)
+{
+    const lbm_config& c = e->cfg;
+    if ((int64_t)n_list * c.nx * c.ny <= kSmallSites) return e->variant_small;
+    const auto& vars = step_variants();
+    int vi = e->variant;
+    if (e->variant_forced) return vi;
+    const int s = stream_variant(c.storage);
+    if (e->variant_tuned && vi != s) return vi;
+    vi = e->variant_tuned ? default_variant(c.storage) : vi;
+    if (c.open_x || e->observe || n_steps < 4 || s < 0) return vi;
+    if (!vars[s].supports(make_params(e, e->all_dev, n_list, vars[s].vec, 0, 3))) return vi;
+    const int threads = (c.nx + 127) / 128 * 32;
+    const int64_t blocks = (int64_t)(512 / threads) * 152;
+    const int64_t min_rows = c.collision == 0 ? 8 : 12;
+    return (int64_t)n_list * c.ny >= min_rows * blocks ? s : vi;
 }
 
 int check_sticky(lbm_ensemble* e)
@@ -614,11 +645,18 @@ int launch_chunk(lbm_ensemble* e, int vi, const int32_t* list_dev, int n_list, i
     const StepVariant::Launch launch = launcher(e, v);
     if (!launch) return fail(LBM_ERR_ARG, "the step variant has no open-channel instantiation");
     // the steps of each launch: one, or for a multi-step variant an odd number
-    // of at most v.multi (observables need the state after every step: one)
+    // of at most v.multi (observables need the state after every step: one);
+    // the row-streaming variant takes chunk mod 4 single steps, then an even
+    // number of two-step launches, so that every variant leaves the state in
+    // the buffer that the parity of the step count names
     std::vector<int> first, count;
+    const int singles = v.kind == 3 ? (e->observe ? chunk : chunk % 4) : 0;
     for (int s = 0; s < chunk;) {
         int k = (v.multi > 1 && !e->observe) ? std::min(v.multi, chunk - s) : 1;
-        if (k % 2 == 0) k -= 1;
+        if (v.kind == 3)
+            k = s < singles ? 1 : 2;
+        else if (k % 2 == 0)
+            k -= 1;
         first.push_back(s);
         count.push_back(k);
         s += k;
@@ -626,6 +664,7 @@ int launch_chunk(lbm_ensemble* e, int vi, const int32_t* list_dev, int n_list, i
     auto params = [&](size_t i) {
         StepParams p = make_params(e, list_dev, n_list, v.vec, first[i], v.kind, chunk);
         p.tb_steps = count[i];
+        p.flip = (int32_t)(i & 1);
         return p;
     };
     // an open channel adds the outlet kernel once per chunk, observables their own kernel per step
@@ -685,7 +724,7 @@ int step_list(lbm_ensemble* e, const int32_t* list_dev, const std::vector<int32_
 {
     const auto& vars = step_variants();
     const int n_list = (int)list.size();
-    int vi = variant_for(e, n_list);
+    int vi = variant_for(e, n_list, n_steps);
     if (vars[vi].supports && !vars[vi].supports(make_params(e, list_dev, n_list, vars[vi].vec, 0, vars[vi].kind)))
         vi = (int64_t)n_list * e->cfg.nx * e->cfg.ny <= kSmallSites ? default_variant_small(e->cfg.storage, true)
                                                                      : default_variant(e->cfg.storage);
@@ -1331,6 +1370,7 @@ int lbm_ensemble_set_variant(lbm_ensemble* e, int32_t variant)
     if (variant == -1) {
         e->variant = default_variant(e->cfg.storage);
         e->variant_small = default_variant_small(e->cfg.storage, e->cfg.open_x != 0);
+        e->variant_forced = e->variant_tuned = false;
         return LBM_OK;
     }
     const auto& v = step_variants();
@@ -1339,6 +1379,7 @@ int lbm_ensemble_set_variant(lbm_ensemble* e, int32_t variant)
     if (!launcher(e, v[variant])) return fail(LBM_ERR_ARG, "the variant has no open-channel instantiation");
     e->variant = variant;  // a forced variant runs every step call
     e->variant_small = variant;
+    e->variant_forced = true;
     return LBM_OK;
 }
 
@@ -1388,6 +1429,8 @@ int lbm_ensemble_autotune(lbm_ensemble* e, int32_t* variant)
     if (wide < 0 || small < 0) return cuda_fail(cudaGetLastError(), "lbm_ensemble_autotune trial launch");
     e->variant = wide;
     e->variant_small = small;
+    e->variant_tuned = true;
+    e->variant_forced = false;
     if (variant) *variant = wide;
     return LBM_OK;
 }

@@ -1,0 +1,725 @@
+// Two fused steps per pass over memory, for large ensembles of periodic channels
+// (App. A streaming and collision, twice): a block walks down the rows of a
+// channel, computes step t + 1 of row y + 1 and, from it and the two rows before,
+// step t + 2 of row y, so that a population value is read from HBM once and
+// written once for two steps.  A single step moves 72 bytes per site (FP32) and
+// is bound by HBM; here a site and step move 36 bytes.
+//
+// Thread = 4 consecutive sites, warp = 128 columns, block = a whole row, so the
+// periodic seam needs no halo.  Each warp copies the nine source rows of its
+// columns into its own shared memory two rows ahead (cp.async, 16 bytes a lane).
+// Of the intermediate step a row's later rows need the populations that move up
+// (2, 5, 6) for two rows, kept in the warp's shared memory, the level ones (0, 1,
+// 3) for one row, kept in registers, and those that move down (4, 7, 8) at once;
+// all in the storage format.  The one-site shift in x is a warp shuffle.  The
+// values at the edges of a warp's columns go to its two neighbours through a
+// ring of four rows in shared memory, with an mbarrier per warp and row: warps
+// wait for their neighbours only, and no block barrier is in the row loop (with
+// one, and the rows staged for the block, the warps stood at the barrier for a
+// quarter of their time).  Every wait is bounded; on timeout a warp records the
+// error and returns.
+//
+// A launch cuts the rows of all listed clones into one contiguous span per
+// block; a span recomputes the intermediate step of one row beyond either end.
+// Per site and step the arithmetic, the order of every sum and the storage
+// rounding are the register-staged kernel's, so populations and drag partials
+// are the same bits.
+//
+// 16 warps of 128 registers an SM: about 120 instructions per site and step, of
+// which the packed BGK collision (lbm_pair.cuh) is 45; FP32 BGK then runs at 0.86
+// of the measured copy bandwidth, the other formats are bound by issue slots and
+// latency.  Fewer registers and more warps spill and lose (FP16: 178 GLUPS at 128
+// registers, 171 at 102, 156 at 85).  Measured, single steps / streamed, GLUPS:
+// FP32 BGK 64 x 1024 x 256 94.6 / 158, 256 x 512 x 128 94.4 / 147, 16 x 2048 x 512
+// 93.3 / 160; FP32 central moments 93.6 / 123; FP16 BGK 157 / 185 (64 x 1024 x
+// 256), 159 / 203 (16 x 2048 x 512); FP16 central moments 132 / 138.
+#pragma once
+#include "async_copy.cuh"
+#include "lbm_pair.cuh"
+
+namespace lbm {
+
+constexpr int kStreamV = 4;             // sites per thread
+constexpr int kStreamMaxThreads = 512;  // rows of up to 2048 sites
+constexpr int kStreamStages = 2;        // source rows in flight
+
+// the rows a span [s, s1) of the linear row index (listed clone, y) loads: per
+// clone the rows [ya, yb) it completes and one row beyond either end
+struct StreamWalk {
+    int s, s1, ny;
+    int li, ya, yb;  // the current piece
+    int y, ye;       // the row to load next, the piece's last
+    __device__ bool piece()
+    {
+        if (s >= s1) return false;
+        li = s / ny;
+        ya = s - li * ny;
+        yb = min(ny, ya + (s1 - s));
+        y = max(ya - 1, 0);
+        ye = min(yb, ny - 1);
+        s += yb - ya;
+        return true;
+    }
+    __device__ bool next() { return y++ < ye ? true : piece(); }
+};
+
+// the pulled values of direction Q at a thread's sites from the row's stored
+// values v at the same sites and the value e beyond the warp's columns
+template <int S, bool SCALED, int Q>
+__device__ __forceinline__ void stream_pull(float2 (&g)[9][kStreamV / 2], const Vec<typename Codec<S>::T, kStreamV>& v,
+                                            typename Codec<S>::T e, bool at_edge, float inv_scale)
+{
+    using K = Carry<S, SCALED>;
+    constexpr int V = kStreamV;
+    float d[V];
+#pragma unroll
+    for (int j = 0; j < V; j += 2) {
+        const float2 f = K::in2(&v.e[j], wf(Q), inv_scale);
+        d[j] = f.x;
+        d[j + 1] = f.y;
+    }
+    if constexpr (cx(Q) == 1) {
+        const float n = __shfl_up_sync(0xffffffffu, d[V - 1], 1);
+#pragma unroll
+        for (int j = V - 1; j > 0; --j) d[j] = d[j - 1];
+        d[0] = at_edge ? K::in(e, wf(Q), inv_scale) : n;
+    } else if constexpr (cx(Q) == -1) {
+        const float n = __shfl_down_sync(0xffffffffu, d[0], 1);
+#pragma unroll
+        for (int j = 0; j < V - 1; ++j) d[j] = d[j + 1];
+        d[V - 1] = at_edge ? K::in(e, wf(Q), inv_scale) : n;
+    }
+#pragma unroll
+    for (int i = 0; i < V / 2; ++i) g[Q][i] = make_float2(d[2 * i], d[2 * i + 1]);
+}
+
+// the same without the shift (a wall returns the node's own population)
+template <int S, bool SCALED, int Q>
+__device__ __forceinline__ void stream_own(float2 (&g)[9][kStreamV / 2], const Vec<typename Codec<S>::T, kStreamV>& v,
+                                           float inv_scale)
+{
+#pragma unroll
+    for (int i = 0; i < kStreamV / 2; ++i) g[Q][i] = Carry<S, SCALED>::in2(&v.e[2 * i], wf(Q), inv_scale);
+}
+
+template <int S, bool SCALED>
+__device__ __forceinline__ void stream_store(Vec<typename Codec<S>::T, kStreamV>& o, const float2 (&g)[kStreamV / 2],
+                                             float w, float scale)
+{
+#pragma unroll
+    for (int i = 0; i < kStreamV / 2; ++i) {
+        if constexpr (S == kFP32) {
+            const float2 f = add2(g[i], splat(w));
+            o.e[2 * i] = f.x;
+            o.e[2 * i + 1] = f.y;
+        } else {
+            Carry<S, SCALED>::out2(&o.e[2 * i], g[i].x, g[i].y, w, scale);
+        }
+    }
+}
+
+// the collision of a thread's sites: BGK on pairs (161 against 150 GLUPS
+// without); the central-moment collision one site at a time, since on pairs its
+// constants and temporaries take registers the row loop does not have (96 bytes
+// of spills, 126 against 127 GLUPS at 64 x 1024 x 256, 123 against 134 at 256 x 512 x 128)
+template <int COLL>
+__device__ __forceinline__ void stream_collide(float2 (&g)[9][kStreamV / 2], const StepParams& p)
+{
+    if constexpr (COLL == 0) {
+        collide2<0, kStreamV / 2>(g, p);
+    } else {
+        float f[9][kStreamV];
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+#pragma unroll
+            for (int i = 0; i < kStreamV / 2; ++i) {
+                f[q][2 * i] = g[q][i].x;
+                f[q][2 * i + 1] = g[q][i].y;
+            }
+#pragma unroll
+        for (int j = 0; j < kStreamV; ++j) collide<COLL, kStreamV>(f, j, p);
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+#pragma unroll
+            for (int i = 0; i < kStreamV / 2; ++i) g[q][i] = make_float2(f[q][2 * i], f[q][2 * i + 1]);
+    }
+}
+
+// The sites whose two steps feel the obstacle: whole 4-site groups covering the
+// columns, and the rows, within two sites of it.  The row stream computes them
+// without the obstacle and does not store them; the blocks compute them apart,
+// a chunk of rows at a time, before they stream.  (With the bounce-back inside
+// the stream the blocks that met the obstacle's rows took twice as long as the
+// others: one launch 593 us with and 223 us without an obstacle, 64 x 1024 x 256.)
+//
+// A group is the sites of one thread of the register-staged kernel whose drag
+// partials these are: 4 for FP32, 8 for 16-bit storage.
+template <int S>
+constexpr int kStreamGroup = S == kFP32 ? 4 : 8;
+
+template <int S>
+struct StreamRegion {
+    static constexpr int G = kStreamGroup<S>;
+    int groups;        // groups of a row
+    int g0, ng;        // first group (may be negative: the row is periodic) and their number
+    int l0, nl;        // the same with one group more on either side, for the intermediate step
+    int r0, r1;        // rows
+    __host__ __device__ explicit StreamRegion(const StepParams& p)
+    {
+        groups = p.nx / G;
+        g0 = (p.ox0 - 2 + G) / G - 1;  // ox0 >= 1: rounded down
+        ng = (p.ox1 + 1) / G - g0 + 1;
+        if (ng > groups) {
+            g0 = 0;
+            ng = groups;
+        }
+        l0 = g0 - 1;
+        nl = ng + 2;
+        if (nl > groups) {
+            l0 = 0;
+            nl = groups;
+        }
+        r0 = p.oy0 - 2 > 0 ? p.oy0 - 2 : 0;
+        r1 = p.oy1 + 2 < p.ny ? p.oy1 + 2 : p.ny;
+        if (p.ox1 <= p.ox0) ng = nl = r0 = r1 = 0;
+    }
+    __host__ __device__ int wrap(int g) const { return g < 0 ? g + groups : (g >= groups ? g - groups : g); }
+    __host__ __device__ bool has(int g) const { return wrap(g - g0) < ng; }
+    // shared memory for a chunk of rows: the intermediate step with one row more
+    // on either side, and both steps' drag terms of each group
+    __host__ __device__ size_t bytes(int rows) const
+    {
+        return (9 * (rows + 2) * G * sizeof(typename Codec<S>::T) + 2 * rows * sizeof(float)) * (size_t)nl;
+    }
+    // rows of a chunk: at most about one chunk per SM over all clones (the chunks
+    // go to the first blocks, which are on different SMs; more chunks recompute
+    // more rows: 110 against 105 us per step, 64 x 1024 x 256), at most one group
+    // of the intermediate step per thread, at least 2 rows
+    __host__ __device__ int chunk(int threads, size_t smem, int sms, int clones) const
+    {
+        const int per_clone = sms > clones ? sms / clones : 1;
+        int r = threads / (nl > 0 ? nl * (G / kStreamV) : 1) - 2, even = (r1 - r0 + per_clone - 1) / per_clone;
+        r = r > even ? even : r;
+        r = r < 2 ? 2 : r;
+        r = r > r1 - r0 ? r1 - r0 : r;
+        while (r > 2 && bytes(r) > smem) --r;
+        return r;
+    }
+};
+
+// four sites x .. x + 3 of row y, from stored values at base[q qs + row rs
+// + column]: row y is row yc there, site x column xc, the sites beyond them
+// columns xl and xr.  Streaming with bounce-back, collision, rest state of solid
+// sites; returns the group's momentum exchange with the obstacle so far: where
+// two threads share a group, the odd lane continues the sum of the lane before.
+template <int S, bool SCALED, int COLL>
+__device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (&g)[9][kStreamV / 2], int x, int y,
+                                                   const typename Codec<S>::T* base, int qs, int rs, int yc, int xc,
+                                                   int xl, int xr)
+{
+    using T = typename Codec<S>::T;
+    using K = Carry<S, SCALED>;
+    constexpr int V = kStreamV;
+    uint32_t cols = 0;  // bit i: site x - 1 + i is in the obstacle's columns
+#pragma unroll
+    for (int i = 0; i < V + 2; ++i) cols |= (x - 1 + i >= p.ox0 && x - 1 + i < p.ox1 ? 1u : 0u) << i;
+    // the sites beyond a periodic seam: columns 0 and nx - 1 are never solid
+    auto solid_row = [&](int r) { return r >= p.oy0 && r < p.oy1; };
+    Vec<T, V> v[9];
+    T e[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const int ys = y - cy(q);
+        const bool wall = ys < 0 || ys >= p.ny;  // the wall returns the node's own population
+        const T* r = base + (wall ? opp(q) * qs + yc * rs : q * qs + (yc - cy(q)) * rs);
+        v[q] = *reinterpret_cast<const Vec<T, V>*>(r + xc);
+        if (cx(q) != 0) e[q] = r[wall ? (cx(q) == 1 ? xc : xc + V - 1) : (cx(q) == 1 ? xl : xr)];
+    }
+    float f[9][V];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const bool wall = y - cy(q) < 0 || y - cy(q) >= p.ny;
+        float d[V], n = 0.f;
+#pragma unroll
+        for (int j = 0; j < V; ++j) d[j] = K::in(v[q].e[j], wf(q), p.inv_scale);
+        if (cx(q) != 0) n = K::in(e[q], wf(q), p.inv_scale);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            if (cx(q) == 1)
+                f[q][j] = wall ? d[j] : (j > 0 ? d[j > 0 ? j - 1 : 0] : n);
+            else if (cx(q) == -1)
+                f[q][j] = wall ? d[j] : (j + 1 < V ? d[j + 1 < V ? j + 1 : 0] : n);
+            else
+                f[q][j] = d[j];
+        }
+        if (q > 0 && solid_row(y - cy(q)) && (cols >> (1 - cx(q)) & ((1u << V) - 1u))) {
+            const Vec<T, V> o = *reinterpret_cast<const Vec<T, V>*>(base + opp(q) * qs + yc * rs + xc);
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                if (cols >> (j + 1 - cx(q)) & 1u) f[q][j] = K::in(o.e[j], wf(q), p.inv_scale);
+        }
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i) g[q][i] = make_float2(f[q][2 * i], f[q][2 * i + 1]);
+    }
+    collide2<COLL, V / 2>(g, p);
+    auto sum = [&](float acc) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const bool solid = solid_row(y) && (cols >> (j + 1) & 1u);
+#pragma unroll
+            for (int q = 1; q < 9; ++q) {
+                if (cx(q) == 0) continue;
+                const float gq = j & 1 ? g[q][j / 2].y : g[q][j / 2].x;
+                if (!solid && solid_row(y + cy(q)) && (cols >> (j + 1 + cx(q)) & 1u))
+                    acc += 2.0f * (float)cx(q) * (wf(q) + gq);
+            }
+        }
+        return acc;
+    };
+    float acc = sum(0.f);
+    if constexpr (kStreamGroup<S> > V) {
+        const float before = __shfl_up_sync(0xffffffffu, acc, 1);
+        if (threadIdx.x & 1) acc = sum(before);
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (solid_row(y) && (cols >> (j + 1) & 1u)) (j & 1 ? g[q][j / 2].y : g[q][j / 2].x) = 0.f;  // rest: f = w
+    return acc;
+}
+
+// the groups of rows [lo, hi) that are not wholly solid, numbered row by row:
+// n groups a row, of which [sa, sa + sn) are solid in the obstacle's rows
+struct StreamGroups {
+    int lo, n, sa, sn, below, inside, total;
+    __device__ StreamGroups(const StepParams& p, int lo_, int hi, int n_, int sa_, int sn_)
+        : lo(lo_), n(n_), sa(sa_), sn(sn_)
+    {
+        const int b = min(max(p.oy0 - lo, 0), hi - lo), e = min(max(p.oy1 - lo, 0), hi - lo);
+        below = b * n;
+        inside = (e - b) * (n - sn);
+        total = below + inside + (hi - lo - e) * n;
+        rows_b = b;
+        rows_e = e;
+    }
+    int rows_b, rows_e;
+    __device__ void at(int i, int& y, int& g) const
+    {
+        if (i < below) {
+            y = lo + i / n;
+            g = i % n;
+        } else if (i < below + inside) {
+            i -= below;
+            y = lo + rows_b + i / (n - sn);
+            g = i % (n - sn);
+            if (g >= sa) g += sn;
+        } else {
+            i -= below + inside;
+            y = lo + rows_e + i / n;
+            g = i % n;
+        }
+    }
+};
+
+// both steps of the obstacle's region for every listed clone, in chunks of rows
+// over the blocks, and the drag partials of its rows
+template <int S, bool SCALED, int COLL>
+__device__ __noinline__ void stream_obstacle(const StepParams& p, unsigned char* smem, int R)
+{
+    using T = typename Codec<S>::T;
+    constexpr int V = kStreamV, G = kStreamGroup<S>, H = G / V;  // H threads per group
+    const StreamRegion<S> rg(p);
+    const int nx = p.nx, ny = p.ny, plane = (int)p.plane, tid = threadIdx.x;
+    const int chunks = (rg.r1 - rg.r0 + R - 1) / R, tw = rg.nl * G;
+    T* const tile = reinterpret_cast<T*>(smem);  // [q][row][tw]
+    const int tq = (R + 2) * tw;
+    float* const terms = reinterpret_cast<float*>(smem + (size_t)9 * tq * sizeof(T));  // [step][row][nl]
+    // whole groups of solid sites: at rest, never read
+    const int sg = (p.ox0 + G - 1) / G, sn = max(p.ox1 / G - sg, 0);
+    for (int item = blockIdx.x; item < p.n_list * chunks; item += gridDim.x) {
+        const int c = p.clone_list[item / chunks];
+        const int cur = p.parity[c] ^ p.flip;
+        const T* src = static_cast<const T*>(cur ? p.buf1 : p.buf0) + (int64_t)c * p.clone_stride;
+        T* dst = static_cast<T*>(cur ? p.buf0 : p.buf1) + (int64_t)c * p.clone_stride;
+        const int ra = rg.r0 + item % chunks * R, rb = min(ra + R, rg.r1);
+        const int la = max(ra - 1, 0), lb = min(rb + 1, ny);
+        const StreamGroups first(p, la, lb, rg.nl, sg - rg.l0, sn), second(p, ra, rb, rg.ng, sg - rg.g0, sn);
+        // (whole warps stay in the loops: the drag sums use shuffles)
+        for (int i = tid; (i & ~31) < first.total * H; i += blockDim.x) {
+            int y, gi;
+            first.at(min(i / H, first.total - 1), y, gi);
+            const bool in = i < first.total * H;
+            const int h = i % H * V, x = rg.wrap(rg.l0 + gi) * G + h;
+            float2 g[9][V / 2];
+            const float acc = stream_site_group<S, SCALED, COLL>(p, g, x, y, src, plane, p.pitch, y, x,
+                                                                 x == 0 ? nx - 1 : x - 1, x + V == nx ? 0 : x + V);
+            if (in) {
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    Vec<T, V> o;
+                    stream_store<S, SCALED>(o, g[q], wf(q), p.scale);
+                    *reinterpret_cast<Vec<T, V>*>(tile + q * tq + (y - la) * tw + gi * G + h) = o;
+                }
+                if (h + V == G && y >= ra && y < rb) terms[(y - ra) * rg.nl + gi] = acc;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; (i & ~31) < second.total * H; i += blockDim.x) {
+            int y, gg;
+            second.at(min(i / H, second.total - 1), y, gg);
+            gg += rg.g0;
+            const bool in = i < second.total * H;
+            const int gi = rg.wrap(gg - rg.l0), h = i % H * V, x = rg.wrap(gg) * G + h, lx = gi * G + h;
+            float2 g[9][V / 2];
+            // (beyond the tile's columns only where it is the whole row)
+            const float acc = stream_site_group<S, SCALED, COLL>(p, g, x, y, tile, tq, tw, y - la, lx,
+                                                                 lx == 0 ? tw - 1 : lx - 1, lx + V == tw ? 0 : lx + V);
+            if (in) {
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    Vec<T, V> o;
+                    stream_store<S, SCALED>(o, g[q], wf(q), p.scale);
+                    st_stream<T, V>(dst + q * plane + y * p.pitch + x, o);
+                }
+                if (h + V == G) terms[(R + y - ra) * rg.nl + gi] = acc;
+            }
+        }
+        const int sa = max(ra, p.oy0), sb = min(rb, p.oy1);
+        const int sv = sn * (G / V);
+        for (int i = tid; i < max(sb - sa, 0) * sv; i += blockDim.x)
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                Vec<T, V> o;
+                const float2 rest[V / 2] = {};
+                stream_store<S, SCALED>(o, rest, wf(q), p.scale);
+                st_stream<T, V>(dst + q * plane + (sa + i / sv) * p.pitch + sg * G + i % sv * V, o);
+            }
+        __syncthreads();
+        // the partial of a ring row and segment of 32 groups: the register-staged
+        // kernel's warp sum
+        const int ya = max(ra, p.ry0), yb = min(rb, p.ry1 + 1), nseg = p.rs1 - p.rs0 + 1;
+        for (int i = tid >> 5; i < 2 * max(yb - ya, 0) * nseg; i += blockDim.x >> 5) {
+            const int step = i & 1, y = ya + (i >> 1) / nseg, seg = p.rs0 + (i >> 1) % nseg;
+            const int g = seg * 32 + (tid & 31), gi = rg.wrap(g - rg.l0);
+            const bool solid = y >= p.oy0 && y < p.oy1 && g >= sg && g < sg + sn;
+            float acc = g < rg.groups && rg.has(g) && !solid ? terms[(step * R + y - ra) * rg.nl + gi] : 0.f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if ((tid & 31) == 0)
+                p.partials[((int64_t)c * p.batch_cap + p.step_in_batch + step) * p.n_slots + (y - p.ry0) * nseg + seg -
+                           p.rs0] = acc;
+        }
+        __syncthreads();
+    }
+}
+
+// keeps the compiler from holding the nine plane offsets of the loads and of
+// the stores in registers across the row loop (they cost one instruction each)
+__device__ __forceinline__ int stream_opaque(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
+// 16 or 4 bytes global -> shared, asynchronously (cp.async)
+__device__ __forceinline__ void stream_copy16(void* to, const void* from)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(to)), "l"(from) : "memory");
+}
+__device__ __forceinline__ void stream_copy8(void* to, const void* from)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(to)), "l"(from) : "memory");
+}
+__device__ __forceinline__ void stream_copy4(void* to, const void* from)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(to)), "l"(from) : "memory");
+}
+
+// shared memory of one warp: the staged source rows of its columns, the values
+// beyond its columns, and the populations that move up, for two rows
+template <int S>
+struct StreamWarpSmem {
+    using VT = Vec<typename Codec<S>::T, kStreamV>;
+    VT row[kStreamStages][9][32];
+    uint32_t beyond[kStreamStages][8];  // 4 bytes that hold the value left (1, 5, 8) or right (3, 6, 7) of the columns
+    VT up[2][3][32];  // directions 2, 5, 6 of the intermediate step, by row mod 2
+};
+
+template <int S, bool SCALED, int COLL>
+__global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const __grid_constant__ StepParams p)
+{
+    using T = typename Codec<S>::T;
+    constexpr int V = kStreamV;
+    using VT = Vec<T, V>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    // edge values of the last rows' intermediate step: per row (mod 4) and warp,
+    // directions 3, 6, 7 at the warp's first site and 1, 5, 8 at its last; a
+    // warp arrives on edge_ready when a row's values are in place
+    __shared__ T edge[4][6][kStreamMaxThreads / 32];
+    __shared__ __align__(8) uint64_t edge_ready[4][kStreamMaxThreads / 32];
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
+    StreamWarpSmem<S>& ws = reinterpret_cast<StreamWarpSmem<S>*>(smem)[warp];
+    const int nx = p.nx, ny = p.ny;
+    const StreamRegion<S> rg(p);
+    // an even share of the rows; a chunk of the obstacle's region takes a block
+    // about as long as two of its rows
+    const int rows = p.n_list * ny, grid = gridDim.x, bytes = nwarp * (int)sizeof(StreamWarpSmem<S>);
+    const int chunk = rg.ng > 0 ? rg.chunk(blockDim.x, bytes, grid / (kStreamMaxThreads / blockDim.x), p.n_list) : 1;
+    const int items = p.n_list * ((rg.r1 - rg.r0 + chunk - 1) / chunk), cost = rows >= 4 * grid ? 2 : 0;
+    auto span = [&](int b) {
+        return (int)((rows + (int64_t)cost * items) * b / grid) - cost * (items / grid * b + min(b, items % grid));
+    };
+    const int s0 = span(blockIdx.x), s1 = span(blockIdx.x + 1);
+    const int x0 = tid * V;
+    const bool active = x0 < nx;
+    const int xr = active ? x0 : nx - V;
+    const bool first = lane == 0, last = lane == 31 || x0 + V >= nx;  // sites at the edges of the warp's columns
+    const int wl = warp == 0 ? nwarp - 1 : warp - 1, wr = warp + 1 == nwarp ? 0 : warp + 1;
+    const bool apart = rg.ng > 0 && rg.has(x0 / kStreamGroup<S>);  // in the obstacle's columns: computed by stream_obstacle
+
+    if (tid < 4 * nwarp) mbar_init(smem_addr(&edge_ready[tid & 3][tid >> 2]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    __syncthreads();
+    if (rg.ng > 0) stream_obstacle<S, SCALED, COLL>(p, smem, chunk);
+
+    StreamWalk w{s0, s1, ny};
+    if (!w.piece()) return;
+    StreamWalk pw = w;  // position of the next row to load
+    bool more = true;
+    auto source = [&](int li) {  // the state the launch reads, of the listed clone li
+        const int c = p.clone_list[li];
+        return static_cast<const T*>((p.parity[c] ^ p.flip) ? p.buf1 : p.buf0) + (int64_t)c * p.clone_stride;
+    };
+    const T* from_clone = source(w.li);
+    // lanes 0..5: the direction whose value beyond the warp's columns the lane
+    // fetches, and that value's column (16-bit: the 4 bytes that hold it)
+    const int eq = lane == 0 ? 1 : lane == 1 ? 5 : lane == 2 ? 8 : lane == 3 ? 3 : lane == 4 ? 6 : 7;
+    const int xw = warp * 32 * V;
+    const int xe = lane < 3 ? (xw == 0 ? nx - 1 : xw - 1) : (xw + 32 * V >= nx ? 0 : xw + 32 * V);
+    auto load_row = [&](int stage) {
+        if (more) {
+            const T* src = from_clone;
+            const int plane = stream_opaque((int)p.plane);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                // the wall returns the population that left this node
+                const bool wall = cy(q) != 0 && (cy(q) == 1 ? pw.y == 0 : pw.y == ny - 1);
+                const T* from = src + (wall ? opp(q) * plane + pw.y * p.pitch : q * plane + (pw.y - cy(q)) * p.pitch) + xr;
+                if constexpr (sizeof(VT) == 16)
+                    stream_copy16(&ws.row[stage][q][lane], from);
+                else
+                    stream_copy8(&ws.row[stage][q][lane], from);
+            }
+            if (lane < 6) {  // at a wall the pull has no shift and the value is not used
+                const int ey = eq == 5 || eq == 6 ? 1 : (eq == 7 || eq == 8 ? -1 : 0);
+                const int sy = min(max(pw.y - ey, 0), ny - 1);
+                const T* from = src + eq * plane + sy * p.pitch + xe;
+                stream_copy4(&ws.beyond[stage][lane], reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(from) & ~uintptr_t(3)));
+            }
+            const int li = pw.li;
+            more = pw.next();
+            if (more && pw.li != li) from_clone = source(pw.li);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    for (int i = 0; i < kStreamStages; ++i) load_row(i);
+    auto beyond = [&](int stage, int i) {
+        const int off = sizeof(T) == 2 ? ((i < 3 ? (xw == 0 ? nx - 1 : xw - 1) : 0) & 1) : 0;
+        return reinterpret_cast<const T*>(&ws.beyond[stage][i])[off];
+    };
+
+    int stage = 0;
+    uint32_t k = 0;  // rows so far: ring position k mod 4, pass k / 4
+    VT B0{}, B1{}, B3{};
+    do {
+        const int c = p.clone_list[w.li];
+        const int cur = p.parity[c] ^ p.flip;
+        T* dst = static_cast<T*>(cur ? p.buf0 : p.buf1) + (int64_t)c * p.clone_stride;
+        for (int y1 = w.y; y1 <= w.yb; ++y1, ++k) {
+            VT C0, C1, C2, C3, C4, C5, C6, C7, C8;
+            const int slot = k & 3;
+            const bool real = y1 < ny;  // beyond the last row only its second step remains
+            if (real) {
+                // ---- first step of row y1
+                asm volatile("cp.async.wait_group %0;\n" ::"n"(kStreamStages - 1) : "memory");
+                __syncwarp();
+                float2 g[9][V / 2];
+                const auto& r = ws.row[stage];
+                T e1{}, e5{}, e8{}, e3{}, e6{}, e7{};
+                if (first) {
+                    e1 = beyond(stage, 0);
+                    e5 = beyond(stage, 1);
+                    e8 = beyond(stage, 2);
+                }
+                if (last) {
+                    e3 = beyond(stage, 3);
+                    e6 = beyond(stage, 4);
+                    e7 = beyond(stage, 5);
+                }
+                stream_pull<S, SCALED, 0>(g, r[0][lane], T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 2>(g, r[2][lane], T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 4>(g, r[4][lane], T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 1>(g, r[1][lane], e1, first, p.inv_scale);
+                stream_pull<S, SCALED, 5>(g, r[5][lane], e5, first, p.inv_scale);
+                stream_pull<S, SCALED, 8>(g, r[8][lane], e8, first, p.inv_scale);
+                stream_pull<S, SCALED, 3>(g, r[3][lane], e3, last, p.inv_scale);
+                stream_pull<S, SCALED, 6>(g, r[6][lane], e6, last, p.inv_scale);
+                stream_pull<S, SCALED, 7>(g, r[7][lane], e7, last, p.inv_scale);
+                if (y1 == 0) {  // walls: the node's own populations come back, unshifted
+                    stream_own<S, SCALED, 5>(g, r[5][lane], p.inv_scale);
+                    stream_own<S, SCALED, 6>(g, r[6][lane], p.inv_scale);
+                }
+                if (y1 == ny - 1) {
+                    stream_own<S, SCALED, 7>(g, r[7][lane], p.inv_scale);
+                    stream_own<S, SCALED, 8>(g, r[8][lane], p.inv_scale);
+                }
+                __syncwarp();
+                load_row(stage);  // every lane has read the stage
+                stage = stage + 1 == kStreamStages ? 0 : stage + 1;
+                stream_collide<COLL>(g, p);
+                auto store = [&](VT& o, int q) { stream_store<S, SCALED>(o, g[q], wf(q), p.scale); };
+                store(C0, 0);
+                store(C1, 1);
+                store(C2, 2);
+                store(C3, 3);
+                store(C4, 4);
+                store(C5, 5);
+                store(C6, 6);
+                store(C7, 7);
+                store(C8, 8);
+                if (first) {
+                    edge[slot][0][warp] = C3.e[0];
+                    edge[slot][1][warp] = C6.e[0];
+                    edge[slot][2][warp] = C7.e[0];
+                }
+                if (last && active) {
+                    edge[slot][3][warp] = C1.e[V - 1];
+                    edge[slot][4][warp] = C5.e[V - 1];
+                    edge[slot][5][warp] = C8.e[V - 1];
+                }
+                __syncwarp();
+            } else {  // the top wall returns the last row's own 2, 5, 6 in directions 4, 7, 8
+                C4 = ws.up[(k + 1) & 1][0][lane];
+                C7 = ws.up[(k + 1) & 1][1][lane];
+                C8 = ws.up[(k + 1) & 1][2][lane];
+            }
+            const VT A2 = ws.up[k & 1][0][lane], A5 = ws.up[k & 1][1][lane], A6 = ws.up[k & 1][2][lane];
+            if (real) {
+                ws.up[k & 1][0][lane] = C2;
+                ws.up[k & 1][1][lane] = C5;
+                ws.up[k & 1][2][lane] = C6;
+            }
+            // the neighbours' edge values of this row.  A warp that waits here
+            // has seen its neighbours finish the row before last, so the ring of
+            // four rows is never overwritten early.
+            if (lane == 0) mbar_arrive(smem_addr(&edge_ready[slot][warp]));
+            const bool ok = mbar_wait_cycles(smem_addr(&edge_ready[slot][wl]), (k >> 2) & 1u, kWaitCycles) &&
+                            mbar_wait_cycles(smem_addr(&edge_ready[slot][wr]), (k >> 2) & 1u, kWaitCycles);
+            if (!__all_sync(0xffffffffu, ok)) {  // a wait ran out: report it and leave, after the copies in flight
+                if (lane == 0 && p.err_flag) atomicExch(p.err_flag, 1);
+                asm volatile("cp.async.wait_all;\n" ::: "memory");
+                return;
+            }
+            const int yo = y1 - 1;
+            if (yo >= w.ya) {
+                // ---- second step of row yo
+                const int sm1 = (slot + 3) & 3, sm2 = (slot + 2) & 3;
+                float2 g[9][V / 2];
+                T e1{}, e5{}, e8{}, e3{}, e6{}, e7{};
+                if (first) {
+                    e1 = edge[sm1][3][wl];
+                    e5 = edge[sm2][4][wl];
+                    e8 = edge[slot][5][wl];
+                }
+                if (last) {
+                    e3 = edge[sm1][0][wr];
+                    e6 = edge[sm2][1][wr];
+                    e7 = edge[slot][2][wr];
+                }
+                stream_pull<S, SCALED, 0>(g, B0, T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 2>(g, A2, T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 4>(g, C4, T(), false, p.inv_scale);
+                stream_pull<S, SCALED, 1>(g, B1, e1, first, p.inv_scale);
+                stream_pull<S, SCALED, 5>(g, A5, e5, first, p.inv_scale);
+                stream_pull<S, SCALED, 8>(g, C8, e8, first, p.inv_scale);
+                stream_pull<S, SCALED, 3>(g, B3, e3, last, p.inv_scale);
+                stream_pull<S, SCALED, 6>(g, A6, e6, last, p.inv_scale);
+                stream_pull<S, SCALED, 7>(g, C7, e7, last, p.inv_scale);
+                if (yo == 0) {  // A holds the row's own 4, 7, 8
+                    stream_own<S, SCALED, 5>(g, A5, p.inv_scale);
+                    stream_own<S, SCALED, 6>(g, A6, p.inv_scale);
+                }
+                if (yo == ny - 1) {  // C holds the row's own 2, 5, 6
+                    stream_own<S, SCALED, 7>(g, C7, p.inv_scale);
+                    stream_own<S, SCALED, 8>(g, C8, p.inv_scale);
+                }
+                stream_collide<COLL>(g, p);
+                if (active && !(apart && yo >= rg.r0 && yo < rg.r1)) {
+                    const int plane = stream_opaque((int)p.plane);
+                    T* out = dst + yo * p.pitch + x0;
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) {
+                        VT o;
+                        stream_store<S, SCALED>(o, g[q], wf(q), p.scale);
+                        st_stream<T, V>(out + q * plane, o);
+                    }
+                }
+            }
+            if (real) {
+                if (y1 == 0) {  // the bottom wall returns row 0's own 4, 7, 8 in directions 2, 5, 6
+                    ws.up[(k + 1) & 1][0][lane] = C4;
+                    ws.up[(k + 1) & 1][1][lane] = C7;
+                    ws.up[(k + 1) & 1][2][lane] = C8;
+                }
+                B0 = C0;
+                B1 = C1;
+                B3 = C3;
+            }
+        }
+    } while (w.piece());
+}
+
+// whole rows of at most 2048 sites in a block; periodic channels
+template <int S>
+bool stream_supported(const StepParams& p)
+{
+    const int threads = (p.nx + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
+    const StreamRegion<S> rg(p);
+    return rg.bytes(2) <= threads / 32 * sizeof(StreamWarpSmem<S>) && !p.open && p.nx % kStreamGroup<S> == 0 && threads <= kStreamMaxThreads &&
+           (int64_t)p.n_list * p.ny < ((int64_t)1 << 31);
+}
+
+template <int S, bool SCALED, int COLL>
+cudaError_t launch_stream_kernel(const StepParams& p, cudaStream_t s)
+{
+    const int threads = (p.nx + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
+    const int ctas = kStreamMaxThreads / threads;  // per SM: the 512 threads that 128 registers leave room for
+    const size_t smem = threads / 32 * sizeof(StreamWarpSmem<S>);
+    int sms = 152, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t rows = (int64_t)p.n_list * p.ny;
+    const int grid = (int)(rows < (int64_t)ctas * sms ? rows : (int64_t)ctas * sms);
+    const cudaError_t e = cudaFuncSetAttribute(step_stream_kernel<S, SCALED, COLL>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(kStreamMaxThreads / 32 * sizeof(StreamWarpSmem<S>)));
+    if (e != cudaSuccess) return e;
+    step_stream_kernel<S, SCALED, COLL><<<grid, threads, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+// one launch of two steps, or of a single one by the register-staged kernel
+// with the same drag segments
+template <int S>
+cudaError_t launch_stream(const StepParams& p, cudaStream_t s)
+{
+    if (p.tb_steps == 1) return launch_step<S, kStreamGroup<S>, 4>(p, s);
+    if (!stream_supported<S>(p) || p.tb_steps != 2) return cudaErrorInvalidValue;
+    const bool scaled = S != kFP32 && p.scale != 1.0f;
+    if (p.coll == 1)
+        return scaled ? launch_stream_kernel<S, S != kFP32, 1>(p, s) : launch_stream_kernel<S, false, 1>(p, s);
+    return scaled ? launch_stream_kernel<S, S != kFP32, 0>(p, s) : launch_stream_kernel<S, false, 0>(p, s);
+}
+
+}  // namespace lbm

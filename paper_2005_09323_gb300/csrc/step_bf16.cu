@@ -1,6 +1,7 @@
 // Instantiations of the fused step for bf16 population storage.
 #include "lbm_step.cuh"
 #include "lbm_step_rows.cuh"
+#include "lbm_step_stream.cuh"
 #include "lbm_step_tb.cuh"
 
 namespace lbm {
@@ -18,6 +19,9 @@ void register_step_bf16(std::vector<StepVariant>& out)
     // several steps per launch from shared memory: the small calls of one AMS branch
     out.push_back({kBF16, 1, kTbThreads / 32, &launch_tb<kBF16>, 2, &tb_supported<kBF16>});
     out.back().multi = kTbHalo;
+    // two steps per pass over memory: large ensembles
+    out.push_back({kBF16, kStreamGroup<kBF16>, kStreamMaxThreads / 32, &launch_stream<kBF16>, 3, &stream_supported<kBF16>});
+    out.back().multi = 2;
 }
 
 }  // namespace lbm

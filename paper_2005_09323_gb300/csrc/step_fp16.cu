@@ -1,6 +1,7 @@
 // Instantiations of the fused step for fp16 population storage.
 #include "lbm_step.cuh"
 #include "lbm_step_rows.cuh"
+#include "lbm_step_stream.cuh"
 #include "lbm_step_tb.cuh"
 
 namespace lbm {
@@ -18,6 +19,9 @@ void register_step_fp16(std::vector<StepVariant>& out)
     // several steps per launch from shared memory: the small calls of one AMS branch
     out.push_back({kFP16, 1, kTbThreads / 32, &launch_tb<kFP16>, 2, &tb_supported<kFP16>});
     out.back().multi = kTbHalo;
+    // two steps per pass over memory: large ensembles
+    out.push_back({kFP16, kStreamGroup<kFP16>, kStreamMaxThreads / 32, &launch_stream<kFP16>, 3, &stream_supported<kFP16>});
+    out.back().multi = 2;
 }
 
 }  // namespace lbm

@@ -1,6 +1,7 @@
 // Instantiations of the fused step for fp32 population storage.
 #include "lbm_step.cuh"
 #include "lbm_step_rows.cuh"
+#include "lbm_step_stream.cuh"
 #include "lbm_step_tb.cuh"
 
 namespace lbm {
@@ -32,6 +33,9 @@ void register_step_fp32(std::vector<StepVariant>& out)
     // several steps per launch from shared memory: the small calls of one AMS branch
     out.push_back({kFP32, 1, kTbThreads / 32, &launch_tb<kFP32>, 2, &tb_supported<kFP32>});
     out.back().multi = kTbHalo;
+    // two steps per pass over memory: large ensembles
+    out.push_back({kFP32, kStreamGroup<kFP32>, kStreamMaxThreads / 32, &launch_stream<kFP32>, 3, &stream_supported<kFP32>});
+    out.back().multi = 2;
 }
 
 }  // namespace lbm

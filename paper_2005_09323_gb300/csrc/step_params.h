@@ -113,7 +113,10 @@ struct StepParams {
     int32_t outlet_from_u;      // 1: the pulls from the outlet column use the outlet computed from
                                 // open_u_prev (the previous step left that column unwritten)
     int32_t write_outlet;       // 1: the launch also writes the outlet column (the chunk's last step)
-    int32_t tb_steps;           // steps of one launch of the temporally blocked kernel (odd)
+    int32_t tb_steps;           // steps of one launch: odd for the temporally blocked kernel, 1 or 2 for the
+                                // row-streaming one
+    int32_t flip;               // row-streaming kernel: launches of the batch before this one, mod 2 (the
+                                // other kernels run an odd number of steps per launch and use step_in_batch)
 };
 
 // consumer warps of the row-staged step kernel; each writes its own drag

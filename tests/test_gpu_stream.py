@@ -1,0 +1,89 @@
+"""The row-streaming step (two steps per pass over memory) against the
+register-staged step with the same drag segments: the same arithmetic in the
+same order, so populations and drag agree bit for bit (no tolerance).  Sizes at
+the edges: one warp and sixteen, a last warp of few sites, two-row channels'
+neighbours, obstacles at the seam, on a wall, one cell large and over most of a
+row, and step counts with every remainder modulo four."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # clones, nx, ny, obstacle, step counts
+    (3, 200, 37, (60, 11, 9, 14), (4, 5, 6, 7)),
+    (5, 8, 5, (0, 0, 0, 0), (8,)),
+    (2, 16, 4, (4, 0, 4, 2), (12,)),
+    (4, 2048, 65, (500, 28, 64, 36), (13,)),
+    (40, 512, 17, (126, 5, 4, 4), (9,)),
+    (2, 64, 20, (1, 3, 20, 4), (8,)),
+    (2, 72, 20, (60, 5, 11, 3), (12,)),
+    (3, 136, 9, (1, 1, 1, 1), (16,)),
+]
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_2005_09323_gb300 import build, lbmrare
+    build.build()
+    lbmrare.lib()
+    return lbmrare
+
+
+def variant(L, storage, kind):
+    """the streaming variant, or the register-staged one of its vector width with four warps"""
+    st = L.STORAGE[storage]
+    vec = 4 if storage == "fp32" else 8
+    for v in range(L.lbm_step_variant_count()):
+        s, ve, warps = L.lbm_step_variant_info(v)
+        if s == st and L.lbm_step_variant_kind(v) == kind and ve == vec and (kind != 0 or warps == 4):
+            return v
+    raise AssertionError("variant not compiled")
+
+
+def run(L, cfg, n, steps, v=None):
+    e = L.lbm_ensemble_create(cfg, n, 5, torch.cuda.current_stream())
+    try:
+        if v is not None:
+            L.lbm_ensemble_set_variant(e, v)
+        l0 = L.lbm_launch_count()
+        for s in steps:
+            L.lbm_ensemble_step(e, s)
+        launches = L.lbm_launch_count() - l0
+        drag = np.zeros((n, sum(steps)))
+        L.lbm_ensemble_drag(e, 0, sum(steps), drag)
+        pops = [L.lbm_ensemble_get_populations(e, c, cfg.nx, cfg.ny) for c in sorted({0, n // 2, n - 1})]
+        return drag, pops, launches
+    finally:
+        L.lbm_ensemble_destroy(e)
+
+
+@pytest.mark.parametrize("storage,shift", [("fp32", 0), ("fp16", 3), ("bf16", 0)])
+@pytest.mark.parametrize("collision", ["bgk", "cm"])
+def test_stream_is_the_single_step_bit_for_bit(L, storage, shift, collision):
+    for n, nx, ny, ob, steps in SHAPES:
+        cfg = L.config(nx, ny, obstacle=ob, tau=0.56, gx=2e-6, gy=-1e-6, storage=storage, shift_exp=shift, max_steps=64,
+                       collision=collision, omega_bulk=1.1, omega_3=0.9, omega_4=1.2)
+        a, b = (run(L, cfg, n, steps, variant(L, storage, k)) for k in (0, 3))
+        assert np.array_equal(a[0], b[0]), (nx, ny)
+        assert all(np.array_equal(x, y) for x, y in zip(a[1], b[1])), (nx, ny)
+
+
+def test_default_streams_large_calls_only(L):
+    """48 clones of 512 x 128 (10 rows a block) stream: 8 steps in 4 launches, as
+    the single steps bit for bit; 16 clones step singly; so does a call of three
+    steps, and every call while observables are recorded"""
+    kw = dict(nx=512, ny=128, obstacle=(120, 56, 16, 16), tau=0.505, gx=1e-6, max_steps=64)
+    drag, pops, launches = run(L, L.config(**kw), 48, (8, 3))
+    assert launches == 4 + 1 + 3 + 1
+    ref = run(L, L.config(**kw), 48, (8, 3), variant(L, "fp32", 0))
+    assert np.array_equal(drag, ref[0]) and all(np.array_equal(x, y) for x, y in zip(pops, ref[1]))
+    assert run(L, L.config(**kw), 16, (8,))[2] == 8 + 1
+    e = L.lbm_ensemble_create(L.config(**kw), 48, 5, torch.cuda.current_stream())
+    try:
+        L.lbm_ensemble_set_observables(e, True)
+        l0 = L.lbm_launch_count()
+        L.lbm_ensemble_step(e, 8)
+        assert L.lbm_launch_count() - l0 == 8 + 8 + 1
+    finally:
+        L.lbm_ensemble_destroy(e)
