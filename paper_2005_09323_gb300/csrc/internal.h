@@ -101,7 +101,11 @@ struct lbm_ensemble {
     void* snaps;
     int32_t perturb_mode;     // coefficients alpha_n: 0 uniform in [0, 1) (App. D); 1 centred, minus 1/2
     double* snap_mass;        // [n_snapshots]
+    double* snap_partials;    // [n_snapshots][red_blocks][3]: block sums of the snapshots' masses
+    void* perturb_coef;       // [N] coefficients of a perturbation launch (lbm_ensemble.cu)
     int32_t n_snaps_set;
+    void* stat_ws;            // workspace of the drag statistics (stats.cu), grown on demand
+    size_t stat_bytes;
     // AMS checkpoints every ckpt_stride steps: [N][n_ckpt] states
     void* ckpt;
     int32_t n_ckpt;

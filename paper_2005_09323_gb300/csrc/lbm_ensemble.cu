@@ -12,6 +12,7 @@
 
 #include "internal.h"
 #include "lbm_device.cuh"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 
@@ -168,7 +169,12 @@ __global__ void window_sum_kernel(const double* drag, int32_t max_steps, int32_t
 }
 
 // F(t) = (1/W) sum_{s=t-W+1}^{t} D(s); thread i owns a contiguous range of t,
-// opens it with a direct sum and slides the window across it.
+// opens it with the sum of its first window and slides the window across it.
+// The opening sums take whole blocks of steps from a table that the thread block
+// fills first: about W / 32 + 32 additions each instead of W (FP64 additions run
+// at two a clock and SM here: 111 us for 64 x 6500 steps and W = 1000 without).
+constexpr int kScoreTable = 2048;
+
 __global__ void scores_kernel(const double* drag, int32_t max_steps, int32_t window, int32_t t_begin, int32_t t_end,
                               double* scores, double* out_max)
 {
@@ -179,12 +185,26 @@ __global__ void scores_kernel(const double* drag, int32_t max_steps, int32_t win
     const int first = t_begin + window, count = t_end - first + 1;
     double best = -INFINITY;
     if (count > 0) {
+        __shared__ double table[kScoreTable];
+        const int len = t_end - t_begin;                                    // steps t_begin + 1 .. t_end
+        const int B = max(32, (len + kScoreTable - 1) / kScoreTable);       // steps of a block
+        const double* r = d + t_begin;                                      // r[i] = D(t_begin + 1 + i)
+        for (int k = threadIdx.x; k * B < len; k += kRedThreads) {
+            double acc = 0.0;
+            for (int i = k * B; i < min(k * B + B, len); ++i) acc += r[i];
+            table[k] = acc;
+        }
+        __syncthreads();
         const int chunk = (count + kRedThreads - 1) / kRedThreads;
         const int ta = first + (int)threadIdx.x * chunk;
         const int tb = min(ta + chunk - 1, t_end);
         if (ta <= tb) {
             double acc = 0.0;
-            for (int s = ta - window + 1; s <= ta; ++s) acc += d[s - 1];
+            int i = ta - window - t_begin;  // the window's steps are r[i] .. r[end - 1]
+            const int end = ta - t_begin;
+            while (i < end && i % B != 0) acc += r[i++];
+            for (; i + B <= end; i += B) acc += table[i / B];
+            while (i < end) acc += r[i++];
             for (int t = ta; t <= tb; ++t) {
                 if (t > ta) acc += d[t - 1] - d[t - window - 1];
                 const double m = acc / (double)window;
@@ -213,146 +233,306 @@ __global__ void first_crossing_kernel(const double* F, int32_t t_lo, int32_t t_h
     if (threadIdx.x == 0) *out = sh[0] == INT32_MAX ? -1 : sh[0];
 }
 
-// Per-block FP64 partial sums of mass and momentum over the fluid nodes of
-// each listed clone (the blocks of one clone cover its sites in a fixed way).
-template <int S>
-__global__ void moments_partial_kernel(const void* buf0, const void* buf1, const int32_t* parity, const int32_t* list,
-                                       int64_t clone_stride, int64_t plane, int32_t pitch, int32_t nx, int32_t ny,
-                                       Solids sol, float inv_scale, double* partial)
+// ---------------------------------------------------------------- masses
+// A sum of FP32 values kept as an unevaluated pair hi + lo (Knuth's two-sum:
+// the rounding error of every addition goes to lo).  A thread adds some sixty
+// values around 1e-2, so the pair carries their sum to about 2^-48 of itself;
+// the sums of the pairs are FP64.  FP64 instructions run at 1/64 of the FP32
+// rate on this GPU: adding every population in FP64, 39 operations a site, took
+// 1537 us for the moments of 64 x 1024 x 256 nodes (0.06 of the copy bandwidth).
+// Two sums side by side, on the packed FP32 instructions.
+struct PairSum {
+    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+    __device__ void add(float2 x)
+    {
+        const float2 s = add2(hi, x), b = sub2(s, hi);
+        lo = add2(lo, add2(sub2(hi, sub2(s, b)), sub2(x, b)));
+        hi = s;
+    }
+    __device__ bool finite() const { return isfinite(hi.x) && isfinite(hi.y); }
+    __device__ double value() const { return ((double)hi.x + (double)hi.y) + ((double)lo.x + (double)lo.y); }
+};
+
+// what a moments launch reads: clone list[i] of an ensemble's buffers, or state
+// i of an array (buf1 and parity null)
+struct StateSource {
+    const void* buf0;
+    const void* buf1;
+    const int32_t* parity;
+    const int32_t* list;
+    int64_t stride, plane;
+    int32_t pitch, nx, ny;
+    __device__ int index(int i) const { return list ? list[i] : i; }
+    template <typename T>
+    __device__ const T* state(int c) const
+    {
+        return static_cast<const T*>(parity && parity[c] ? buf1 : buf0) + (int64_t)c * stride;
+    }
+};
+
+// the states a snapshot bank is filled from (element offsets from one base each)
+struct SnapSources {
+    const void* from[16];
+};
+
+constexpr int kMassVec = 4;  // sites per thread and load
+
+__device__ __forceinline__ uint32_t fluid_bits(const Solids& sol, int x, int y, int nx)
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int j = 0; j < kMassVec; ++j) m |= (x + j < nx && !sol.at(x + j, y) ? 1u : 0u) << j;
+    return m;
+}
+
+// per-block FP64 partial sums over the blocks of each state; fixed order.
+// COPY: the states come from snap.from and are copied to the bank `copy` on the
+// way.  NEEDED: only clones that another slot has for its parent.
+template <int S, bool MOM, bool COPY, bool NEEDED>
+__global__ void __launch_bounds__(kRedThreads) moments_partial_kernel(const StateSource src, const SnapSources snap,
+                                                                      void* copy, const int32_t* parent,
+                                                                      int32_t n_clones, Solids sol, float inv_scale,
+                                                                      double* partial)
 {
     using T = typename Codec<S>::T;
+    using VT = Vec<T, kMassVec>;
     __shared__ double sh[kRedThreads];
-    const int li = blockIdx.y;
-    const int c = list[li];
-    const T* base = static_cast<const T*>(parity[c] ? buf1 : buf0) + (int64_t)c * clone_stride;
-    const int64_t sites = (int64_t)nx * ny;
-    double m = 0.0, px = 0.0, py = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < sites; i += (int64_t)gridDim.x * kRedThreads) {
-        const int y = (int)(i / nx), x = (int)(i - (int64_t)y * nx);
-        if (sol.at(x, y)) continue;
-        const T* cell = base + (int64_t)y * pitch + x;
+    const int c = COPY ? (int)blockIdx.y : src.index(blockIdx.y);
+    if constexpr (NEEDED) {
+        bool used = false;
+        for (int s = threadIdx.x; s < n_clones; s += kRedThreads) used |= s != c && parent[s] == c;
+        if (!__syncthreads_or(used)) return;
+    }
+    const T* base = COPY ? static_cast<const T*>(snap.from[c]) : src.state<T>(c);
+    T* to = COPY ? static_cast<T*>(copy) + (int64_t)c * src.stride : nullptr;
+    // a copy takes the rows' padding along
+    const int gx = (COPY ? src.pitch : (src.nx + kMassVec - 1)) / kMassVec, groups = gx * src.ny;
+    PairSum m, px, py;
+    int count = 0;
+    for (int i = blockIdx.x * kRedThreads + threadIdx.x; i < groups; i += gridDim.x * kRedThreads) {
+        const int y = i / gx, x = (i - y * gx) * kMassVec;
+        const int64_t off = (int64_t)y * src.pitch + x;
+        VT v[9];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const double f = (double)wf(q) + (double)Codec<S>::dec(cell[q * plane], wf(q), inv_scale);
-            m += f;
-            px += cx(q) * f;
-            py += cy(q) * f;
+        for (int q = 0; q < 9; ++q) v[q] = *reinterpret_cast<const VT*>(base + q * src.plane + off);
+        if constexpr (COPY) {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) *reinterpret_cast<VT*>(to + q * src.plane + off) = v[q];
+        }
+        const uint32_t fluid = fluid_bits(sol, x, y, src.nx);
+        count += __popc(fluid);
+        // without the rest weights; sites outside the fluid add zeros
+#pragma unroll
+        for (int j = 0; j < kMassVec; j += 2)
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                float2 g = Codec<S>::dec2(&v[q].e[j], wf(q), inv_scale);
+                g.x = fluid >> j & 1u ? g.x : 0.f;
+                g.y = fluid >> (j + 1) & 1u ? g.y : 0.f;
+                m.add(g);
+                const float2 n = make_float2(-g.x, -g.y);
+                if (MOM && cx(q) != 0) px.add(cx(q) > 0 ? g : n);
+                if (MOM && cy(q) != 0) py.add(cy(q) > 0 ? g : n);
+            }
+    }
+    constexpr double kRest = 4.0 * (double)wf(1) + 4.0 * (double)wf(5) + (double)wf(0);
+    double dm = m.value() + kRest * count, dx = px.value(), dy = py.value();
+    if (!m.finite() || !px.finite() || !py.finite()) {  // beyond FP32's range: this thread's sites in FP64
+        dm = dx = dy = 0.0;
+        for (int i = blockIdx.x * kRedThreads + threadIdx.x; i < groups; i += gridDim.x * kRedThreads) {
+            const int y = i / gx, x = (i - y * gx) * kMassVec;
+            const uint32_t fluid = fluid_bits(sol, x, y, src.nx);
+            for (int j = 0; j < kMassVec; ++j)
+                for (int q = 0; q < 9 && (fluid >> j & 1u); ++q) {
+                    const double f = (double)wf(q) + (double)Codec<S>::dec(
+                                                         base[q * src.plane + (int64_t)y * src.pitch + x + j], wf(q), inv_scale);
+                    dm += f;
+                    dx += cx(q) * f;
+                    dy += cy(q) * f;
+                }
         }
     }
-    const double sm = block_sum<kRedThreads>(m, sh);
-    const double sx = block_sum<kRedThreads>(px, sh);
-    const double sy = block_sum<kRedThreads>(py, sh);
+    dm = block_sum<kRedThreads>(dm, sh);
+    if (MOM) {
+        dx = block_sum<kRedThreads>(dx, sh);
+        dy = block_sum<kRedThreads>(dy, sh);
+    }
     if (threadIdx.x == 0) {
         double* o = partial + ((int64_t)c * gridDim.x + blockIdx.x) * 3;
-        o[0] = sm; o[1] = sx; o[2] = sy;
+        o[0] = dm;
+        o[1] = dx;
+        o[2] = dy;
     }
 }
+
+// the sum of a state's block partials (component k), by a whole block in a fixed order
+template <int THREADS>
+__device__ double partial_sum(const double* partial, int64_t c, int32_t nblocks, int k, double* sh)
+{
+    double v = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += THREADS) v += partial[(c * nblocks + b) * 3 + k];
+    return block_sum<THREADS>(v, sh);
+}
+
+constexpr int kFinalThreads = 256;
 
 __global__ void moments_final_kernel(const double* partial, int32_t nblocks, const int32_t* list, double* mass,
                                      double* px, double* py)
 {
-    const int c = list[blockIdx.x];
-    if (threadIdx.x != 0) return;
-    double m = 0, x = 0, y = 0;
-    for (int b = 0; b < nblocks; ++b) {
-        const double* o = partial + ((int64_t)c * nblocks + b) * 3;
-        m += o[0]; x += o[1]; y += o[2];
+    __shared__ double sh[kFinalThreads];
+    const int c = list ? list[blockIdx.x] : (int)blockIdx.x;
+    double* const out[3] = {mass, px, py};
+    for (int k = 0; k < 3; ++k) {
+        if (!out[k]) continue;
+        const double v = partial_sum<kFinalThreads>(partial, c, nblocks, k, sh);
+        if (threadIdx.x == 0) out[k][c] = v;
     }
-    mass[c] = m;
-    if (px) px[c] = x;
-    if (py) py[c] = y;
 }
 
-// fluid mass of every state in the snapshot bank (fixed-order FP64 partials)
-template <int S>
-__global__ void bank_mass_partial_kernel(const void* snaps, int64_t clone_stride, int64_t plane, int32_t pitch,
-                                         int32_t nx, int32_t ny, Solids sol, float inv_scale, double* partial)
-{
-    using T = typename Codec<S>::T;
-    __shared__ double sh[kRedThreads];
-    const int k = blockIdx.y;
-    const T* base = static_cast<const T*>(snaps) + (int64_t)k * clone_stride;
-    const int64_t sites = (int64_t)nx * ny;
-    double m = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < sites; i += (int64_t)gridDim.x * kRedThreads) {
-        const int y = (int)(i / nx), x = (int)(i - (int64_t)y * nx);
-        if (sol.at(x, y)) continue;
-        const T* cell = base + (int64_t)y * pitch + x;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) m += (double)wf(q) + (double)Codec<S>::dec(cell[q * plane], wf(q), inv_scale);
-    }
-    const double sm = block_sum<kRedThreads>(m, sh);
-    if (threadIdx.x == 0) partial[(int64_t)k * gridDim.x + blockIdx.x] = sm;
-}
-
-__global__ void bank_mass_final_kernel(const double* partial, int32_t nblocks, double* snap_mass)
-{
-    if (threadIdx.x != 0) return;
-    double m = 0.0;
-    for (int b = 0; b < nblocks; ++b) m += partial[(int64_t)blockIdx.x * nblocks + b];
-    snap_mass[blockIdx.x] = m;
-}
-
-// perturb_kernel's `inplace` value that perturbs every listed slot in place
+// ---------------------------------------------------------------- perturbation
+// perturb kernels' `inplace` value that perturbs every listed slot in place
 constexpr int32_t kAllInPlace = -2;
+constexpr int kMaxSnaps = 16;
+
+// one slot's coefficients: eps alpha_n, and the rescale to the parent's mass
+struct PerturbCoef {
+    float alpha_eps[kMaxSnaps];
+    float sm, sm1;     // M_p / (M_p + lin) and that minus 1
+    int32_t from;      // parent, -1: the slot keeps its state
+    int32_t pad;
+};
 
 // App. D: slot s with parent p != s (or s == inplace, or every listed slot
 // with inplace == kAllInPlace) becomes
 //   f_s = (f_p + eps sum_n alpha_n f^(n)) * M_p / (M_p + eps sum_n alpha_n M^(n))
-// on fluid nodes, written in the shifted variable g = f - w.  alpha_n is the
-// counter-based uniform in [0, 1) minus alpha_shift: 0 for the printed form,
-// 1/2 for the centred coefficients (lbm_ensemble_set_perturbation).
-template <int S>
-__global__ void perturb_kernel(void* buf0, void* buf1, const int32_t* parity, const int32_t* parent, int32_t n_clones,
-                               int32_t* flag, int32_t inplace, const int32_t* slots,
-                               int64_t clone_stride, int64_t plane, int32_t pitch, int32_t nx, int32_t ny,
-                               Solids sol, const void* snaps, int32_t n_s,
-                               const double* snap_mass, const double* mass, double eps, uint64_t seed, uint64_t iter,
-                               double alpha_shift, float scale, float inv_scale)
+// on fluid nodes.  alpha_n is the counter-based uniform in [0, 1) minus
+// alpha_shift: 0 for the printed form, 1/2 for the centred coefficients
+// (lbm_ensemble_set_perturbation).  One block per slot: its coefficients, with
+// the parent's mass summed from the partials of the moments launch before.
+__global__ void perturb_coef_kernel(const int32_t* parent, int32_t n_clones, int32_t* flag, int32_t inplace,
+                                    const int32_t* slots, int32_t n_s, const double* snap_mass, const double* partial,
+                                    int32_t nblocks, double eps, uint64_t seed, uint64_t iter, double alpha_shift,
+                                    PerturbCoef* coef)
 {
-    using T = typename Codec<S>::T;
-    const int s = slots ? slots[blockIdx.y] : (int)blockIdx.y;
+    __shared__ double sh[kFinalThreads];
+    __shared__ double alpha[kMaxSnaps];
+    const int s = slots ? slots[blockIdx.x] : (int)blockIdx.x;
     const int p = parent[s];
-    if (p < 0 || p >= n_clones) {  // rejected selection: leave the slot alone
-        if (threadIdx.x == 0) flag[0] = 1;
+    PerturbCoef& out = coef[blockIdx.x];
+    const bool outside = p < 0 || p >= n_clones;  // rejected selection: leave the slot alone
+    if (outside || (p == s && s != inplace && inplace != kAllInPlace)) {
+        if (threadIdx.x == 0) {
+            if (outside) flag[0] = 1;
+            out.from = -1;
+        }
         return;
     }
-    if (p == s && s != inplace && inplace != kAllInPlace) return;  // block-uniform
-    __shared__ float alpha_eps[16];
-    __shared__ float sc_m1[2];
-    if (threadIdx.x == 0) {
-        double lin = 0.0;
-        for (int k = 0; k < n_s; ++k) {
-            const u64x4 r = philox(kStreamPerturb, iter, (uint64_t)s, (uint64_t)k, seed, 0u);
-            const double a = unit_double(r.v[0]) - alpha_shift;
-            alpha_eps[k] = (float)(eps * a);
-            lin += eps * a * snap_mass[k];
-        }
-        const double Mp = mass[p];
-        const double scale_m = eps == 0.0 ? 1.0 : Mp / (Mp + lin);
-        sc_m1[0] = (float)scale_m;
-        sc_m1[1] = (float)(scale_m - 1.0);
+    const double Mp = eps == 0.0 ? 1.0 : partial_sum<kFinalThreads>(partial, p, nblocks, 0, sh);
+    if ((int)threadIdx.x < n_s) {
+        const u64x4 r = philox(kStreamPerturb, iter, (uint64_t)s, (uint64_t)threadIdx.x, seed, 0u);
+        alpha[threadIdx.x] = unit_double(r.v[0]) - alpha_shift;
+        out.alpha_eps[threadIdx.x] = (float)(eps * alpha[threadIdx.x]);
     }
     __syncthreads();
-    const float sm = sc_m1[0], sm1 = sc_m1[1];
-    const T* from = static_cast<const T*>(parity[p] ? buf1 : buf0) + (int64_t)p * clone_stride;
-    T* to = static_cast<T*>(parity[s] ? buf1 : buf0) + (int64_t)s * clone_stride;
-    const T* sn = static_cast<const T*>(snaps);
-    const int64_t sites = (int64_t)nx * ny;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < sites; i += (int64_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / nx), x = (int)(i - (int64_t)y * nx);
-        if (sol.at(x, y)) continue;  // solid: stays at rest
-        const int64_t off = (int64_t)y * pitch + x;
+    if (threadIdx.x == 0) {
+        double lin = 0.0;
+        for (int k = 0; k < n_s; ++k) lin += eps * alpha[k] * snap_mass[k];
+        const double scale_m = eps == 0.0 ? 1.0 : Mp / (Mp + lin);
+        out.sm = (float)scale_m;
+        out.sm1 = (float)(scale_m - 1.0);
+        out.from = p;
+    }
+}
+
+// the perturbed copies.  A thread holds 4 sites of one direction of every
+// snapshot and walks the slots that change among kPerturbSlots, so the bank is
+// read once for them all (HBM bound by the parents and the copies then; with
+// the bank read again for every slot, one site at a time, the copies of 24 of
+// 64 x 1024 x 256 nodes took 557 us against 67 us of such traffic)
+constexpr int kPerturbSlots = 64, kPerturbAhead = 4;
+
+template <int S, int NS>
+__global__ void __launch_bounds__(256) perturb_kernel(void* buf0, void* buf1, const int32_t* parity,
+                                                      const int32_t* slots, int32_t n_slots, int64_t clone_stride,
+                                                      int64_t plane, int32_t pitch, int32_t nx, int32_t ny, Solids sol,
+                                                      const void* snaps, int32_t n_s, const PerturbCoef* coef,
+                                                      float scale, float inv_scale)
+{
+    using T = typename Codec<S>::T;
+    constexpr int V = kMassVec;
+    using VT = Vec<T, V>;
+    __shared__ float c_alpha[kPerturbSlots][NS > 0 ? NS : 1];
+    __shared__ float c_sm[kPerturbSlots], c_sm1[kPerturbSlots];
+    __shared__ const T* c_from[kPerturbSlots];
+    __shared__ T* c_to[kPerturbSlots];
+    __shared__ int n_live;
+    // the slots of this block that change, in order
+    const int first = blockIdx.y * kPerturbSlots, here = min(kPerturbSlots, n_slots - first);
+    if (threadIdx.x < 32) {
+        int live = 0;
+        for (int b = 0; b < here; b += 32) {
+            const int i = b + (int)threadIdx.x;
+            const int from = i < here ? coef[first + i].from : -1;
+            const uint32_t set = __ballot_sync(0xffffffffu, from >= 0);
+            if (from >= 0) {
+                const int k = live + __popc(set & ((1u << threadIdx.x) - 1u)), s = slots ? slots[first + i] : first + i;
+                c_from[k] = static_cast<const T*>(parity[from] ? buf1 : buf0) + (int64_t)from * clone_stride;
+                c_to[k] = static_cast<T*>(parity[s] ? buf1 : buf0) + (int64_t)s * clone_stride;
+                c_sm[k] = coef[first + i].sm;
+                c_sm1[k] = coef[first + i].sm1;
+                for (int j = 0; j < n_s; ++j) c_alpha[k][j] = coef[first + i].alpha_eps[j];
+            }
+            live += __popc(set);
+        }
+        if (threadIdx.x == 0) n_live = live;
+    }
+    __syncthreads();
+    const int live = n_live;
+    if (live == 0) return;
+    const int gx = (nx + V - 1) / V, per_q = gx * ny, i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= 9 * per_q) return;
+    const int q = i / per_q, r = i - q * per_q, y = r / gx, x = (r - y * gx) * V;
+    const uint32_t fluid = fluid_bits(sol, x, y, nx);
+    if (fluid == 0u) return;
+    const int64_t off = q * plane + (int64_t)y * pitch + x;
+    const float w = q == 0 ? wf(0) : (q <= 4 ? wf(1) : wf(5));
+    float sn[NS > 0 ? NS : 1][V];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const float w = wf(q);
-            const float g = Codec<S>::dec(from[q * plane + off], w, inv_scale);
-            float add = 0.f;
-            for (int k = 0; k < n_s; ++k)
-                add += alpha_eps[k] * (w + Codec<S>::dec(sn[(int64_t)k * clone_stride + q * plane + off], w, inv_scale));
-            // f_new - w = (g + add) * sm + w * (sm - 1)
-            const float gn = (g + add) * sm + w * sm1;
-            to[q * plane + off] = Codec<S>::enc(gn, w, scale);
+    for (int k = 0; k < NS; ++k)
+        if (k < n_s) {
+            const VT v = *reinterpret_cast<const VT*>(static_cast<const T*>(snaps) + k * clone_stride + off);
+#pragma unroll
+            for (int j = 0; j < V; ++j) sn[k][j] = w + Codec<S>::dec(v.e[j], w, inv_scale);
+        }
+    for (int l0 = 0; l0 < live; l0 += kPerturbAhead) {
+        VT g[kPerturbAhead];
+#pragma unroll
+        for (int u = 0; u < kPerturbAhead; ++u)
+            if (l0 + u < live) g[u] = *reinterpret_cast<const VT*>(c_from[l0 + u] + off);
+#pragma unroll
+        for (int u = 0; u < kPerturbAhead; ++u) {
+            const int l = l0 + u;
+            if (l >= live) break;
+            const float sm = c_sm[l], sm1 = c_sm1[l];
+            VT o;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                float add = 0.f;
+#pragma unroll
+                for (int k = 0; k < NS; ++k)
+                    if (k < n_s) add += c_alpha[l][k] * sn[k][j];
+                // f_new - w = (g + add) * sm + w * (sm - 1)
+                const float gn = (Codec<S>::dec(g[u].e[j], w, inv_scale) + add) * sm + w * sm1;
+                o.e[j] = Codec<S>::enc(gn, w, scale);
+            }
+            T* to = c_to[l] + off;
+            if (fluid == (1u << V) - 1u) {
+                *reinterpret_cast<VT*>(to) = o;
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (fluid >> j & 1u) to[j] = o.e[j];  // solid nodes stay at rest
+            }
         }
     }
 }
@@ -780,57 +960,104 @@ int step_list(lbm_ensemble* e, const int32_t* list_dev, const std::vector<int32_
     return LBM_OK;
 }
 
-int compute_masses(lbm_ensemble* e, const int32_t* list_dev, int n_list)
+// blocks of a moments launch per state: two 4-site groups for each thread (one
+// each is bound by the FP64 sums of the blocks)
+int moment_blocks(const lbm_ensemble* e)
 {
-    const Solids sol = solids_of(e->cfg);
+    const int64_t groups = (int64_t)((e->cfg.nx + kMassVec - 1) / kMassVec) * e->cfg.ny;
+    return (int)std::min<int64_t>(e->red_blocks, (groups + 2 * kRedThreads - 1) / (2 * kRedThreads));
+}
+
+StateSource ensemble_states(const lbm_ensemble* e, const int32_t* list_dev)
+{
+    return {e->buf[0], e->buf[1], e->parity_dev, list_dev, e->clone_stride, e->plane, e->pitch, e->cfg.nx, e->cfg.ny};
+}
+
+// mass partials of the listed clones; parent_dev != null: of the clones another
+// slot has for its parent only
+int mass_partials(lbm_ensemble* e, const int32_t* list_dev, int n_list, const int32_t* parent_dev)
+{
     return dispatch_storage(e->cfg.storage, [&](auto tag) -> int {
         constexpr int S = decltype(tag)::value;
-        dim3 grid(e->red_blocks, n_list);
-        moments_partial_kernel<S><<<grid, kRedThreads, 0, e->stream>>>(
-            e->buf[0], e->buf[1], e->parity_dev, list_dev, e->clone_stride, e->plane, e->pitch, e->cfg.nx, e->cfg.ny,
-            sol, e->inv_scale, e->red_partials);
-        count_launches(1);
-        LBM_CUDA(cudaGetLastError());
-        moments_final_kernel<<<n_list, 32, 0, e->stream>>>(e->red_partials, e->red_blocks, list_dev, e->mass_dev,
-                                                            e->mass_dev + e->n, e->mass_dev + 2 * e->n);
+        const dim3 grid(moment_blocks(e), n_list);
+        const StateSource src = ensemble_states(e, list_dev);
+        if (parent_dev)
+            moments_partial_kernel<S, false, false, true><<<grid, kRedThreads, 0, e->stream>>>(
+                src, SnapSources{}, nullptr, parent_dev, e->n, solids_of(e->cfg), e->inv_scale, e->red_partials);
+        else
+            moments_partial_kernel<S, false, false, false><<<grid, kRedThreads, 0, e->stream>>>(
+                src, SnapSources{}, nullptr, nullptr, e->n, solids_of(e->cfg), e->inv_scale, e->red_partials);
         count_launches(1);
         LBM_CUDA(cudaGetLastError());
         return LBM_OK;
     });
 }
 
-int bank_masses(lbm_ensemble* e, int n_s)
+// mass and momentum of the listed clones into mass_dev
+int compute_moments(lbm_ensemble* e, const int32_t* list_dev, int n_list)
 {
-    const Solids sol = solids_of(e->cfg);
     return dispatch_storage(e->cfg.storage, [&](auto tag) -> int {
         constexpr int S = decltype(tag)::value;
-        bank_mass_partial_kernel<S><<<dim3(e->red_blocks, n_s), kRedThreads, 0, e->stream>>>(
-            e->snaps, e->clone_stride, e->plane, e->pitch, e->cfg.nx, e->cfg.ny, sol, e->inv_scale,
+        const int blocks = moment_blocks(e);
+        moments_partial_kernel<S, true, false, false><<<dim3(blocks, n_list), kRedThreads, 0, e->stream>>>(
+            ensemble_states(e, list_dev), SnapSources{}, nullptr, nullptr, e->n, solids_of(e->cfg), e->inv_scale,
             e->red_partials);
         LBM_CUDA(cudaGetLastError());
-        bank_mass_final_kernel<<<n_s, 32, 0, e->stream>>>(e->red_partials, e->red_blocks, e->snap_mass);
+        moments_final_kernel<<<n_list, kFinalThreads, 0, e->stream>>>(e->red_partials, blocks, list_dev, e->mass_dev,
+                                                                       e->mass_dev + e->n, e->mass_dev + 2 * e->n);
         LBM_CUDA(cudaGetLastError());
         count_launches(2);
         return LBM_OK;
     });
 }
 
+// fill the App. D bank with n_s states and record their masses, in one pass
+int fill_bank(lbm_ensemble* e, int n_s, const SnapSources& from)
+{
+    return dispatch_storage(e->cfg.storage, [&](auto tag) -> int {
+        constexpr int S = decltype(tag)::value;
+        const int blocks = moment_blocks(e);
+        moments_partial_kernel<S, false, true, false><<<dim3(blocks, n_s), kRedThreads, 0, e->stream>>>(
+            ensemble_states(e, nullptr), from, e->snaps, nullptr, e->n, solids_of(e->cfg), e->inv_scale,
+            e->snap_partials);
+        LBM_CUDA(cudaGetLastError());
+        moments_final_kernel<<<n_s, kFinalThreads, 0, e->stream>>>(e->snap_partials, blocks, nullptr, e->snap_mass,
+                                                                    nullptr, nullptr);
+        LBM_CUDA(cudaGetLastError());
+        count_launches(2);
+        return LBM_OK;
+    });
+}
+
+// the perturbed copies of every slot, or of the n_slots listed ones; the mass
+// partials of the parents must have been launched before when eps != 0
 int run_perturb(lbm_ensemble* e, const int32_t* parent_dev, int32_t inplace, double eps, uint64_t seed, uint64_t iter,
                 const int32_t* slots = nullptr, int32_t n_slots = -1)
 {
-    const Solids sol = solids_of(e->cfg);
-    const int n_s = eps != 0.0 ? e->n_snaps_set : 0;
+    const int n_s = eps != 0.0 ? e->n_snaps_set : 0, n = slots ? n_slots : e->n;
+    perturb_coef_kernel<<<n, kFinalThreads, 0, e->stream>>>(parent_dev, e->n, e->flag_dev, inplace, slots, n_s,
+                                                             e->snap_mass, e->red_partials, moment_blocks(e), eps, seed,
+                                                             iter, e->perturb_mode ? 0.5 : 0.0,
+                                                             static_cast<PerturbCoef*>(e->perturb_coef));
+    LBM_CUDA(cudaGetLastError());
     return dispatch_storage(e->cfg.storage, [&](auto tag) -> int {
         constexpr int S = decltype(tag)::value;
-        const int64_t sites = (int64_t)e->cfg.nx * e->cfg.ny;
-        const int bx = (int)std::min<int64_t>((sites + 255) / 256, 1024);
-        dim3 grid(bx, slots ? n_slots : e->n);
-        perturb_kernel<S><<<grid, 256, 0, e->stream>>>(
-            e->buf[0], e->buf[1], e->parity_dev, parent_dev, e->n, e->flag_dev, inplace, slots, e->clone_stride, e->plane, e->pitch, e->cfg.nx,
-            e->cfg.ny, sol, e->snaps, n_s, e->snap_mass, e->mass_dev, eps, seed, iter,
-            e->perturb_mode ? 0.5 : 0.0, e->scale, e->inv_scale);
-        count_launches(1);
+        const int64_t groups = (int64_t)((e->cfg.nx + kMassVec - 1) / kMassVec) * e->cfg.ny * 9;
+        const dim3 grid((unsigned)((groups + 255) / 256), (n + kPerturbSlots - 1) / kPerturbSlots);
+        auto go = [&](auto snaps) {
+            perturb_kernel<S, decltype(snaps)::value><<<grid, 256, 0, e->stream>>>(
+                e->buf[0], e->buf[1], e->parity_dev, slots, n, e->clone_stride, e->plane, e->pitch, e->cfg.nx,
+                e->cfg.ny, solids_of(e->cfg), e->snaps, n_s, static_cast<const PerturbCoef*>(e->perturb_coef),
+                e->scale, e->inv_scale);
+        };
+        if (n_s == 0)
+            go(std::integral_constant<int, 0>{});
+        else if (n_s <= 10)  // the paper's N_s
+            go(std::integral_constant<int, 10>{});
+        else
+            go(std::integral_constant<int, kMaxSnaps>{});
         LBM_CUDA(cudaGetLastError());
+        count_launches(2);
         return LBM_OK;
     });
 }
@@ -940,7 +1167,9 @@ int lbm_ensemble_create(const lbm_config* cfg, int32_t n_clones, uint64_t seed, 
     ALLOC(e->flag_dev, sizeof(int32_t) * 4);
     ALLOC(e->red_partials, sizeof(double) * 3 * (size_t)n_clones * e->red_blocks);
     ALLOC(e->mass_dev, sizeof(double) * 3 * n_clones);
+    ALLOC(e->perturb_coef, sizeof(PerturbCoef) * n_clones);
     if (c.n_snapshots > 0) {
+        ALLOC(e->snap_partials, sizeof(double) * 3 * c.n_snapshots * e->red_blocks);
         ALLOC(e->snaps, (size_t)e->clone_stride * e->elem_bytes * c.n_snapshots);
         ALLOC(e->snap_mass, sizeof(double) * c.n_snapshots);
     }
@@ -1017,7 +1246,8 @@ int lbm_ensemble_destroy(lbm_ensemble* e)
     void* ptrs[] = {e->buf[0], e->buf[1], e->parity_dev, e->t_dev, e->list_dev, e->all_dev, e->partials,
                     e->drag, e->scores, e->flag_dev, e->red_partials, e->mass_dev, e->snaps, e->snap_mass, e->ckpt,
                     e->fields_list_dev, e->cnn_x, e->cnn_pred, e->cnn_score, e->pot[0], e->pot[1], e->pot[2],
-                    e->pot_tmp[0], e->pot_tmp[1], e->om_col, e->inlet_g, e->open_u, e->obs};
+                    e->pot_tmp[0], e->pot_tmp[1], e->om_col, e->inlet_g, e->open_u, e->obs, e->perturb_coef,
+                    e->snap_partials, e->stat_ws};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete e;
@@ -1145,16 +1375,14 @@ int lbm_ensemble_set_snapshots(lbm_ensemble* e, int32_t n_s, const int32_t* clon
     if (!e || (n_s > 0 && !clones)) return fail(LBM_ERR_ARG, "null argument");
     if (n_s < 0 || n_s > e->cfg.n_snapshots) return fail(LBM_ERR_ARG, "more snapshots than the bank holds");
     const size_t bytes = (size_t)e->clone_stride * e->elem_bytes;
-    std::vector<int32_t> list(clones, clones + n_s);
+    SnapSources from{};
     for (int k = 0; k < n_s; ++k) {
-        const int c = list[k];
+        const int c = clones[k];
         if (c < 0 || c >= e->n) return fail(LBM_ERR_ARG, "clone index out of range");
-        LBM_CUDA(cudaMemcpyAsync(static_cast<char*>(e->snaps) + (size_t)k * bytes,
-                                 static_cast<char*>(e->buf[e->parity_host[c]]) + (size_t)c * bytes, bytes,
-                                 cudaMemcpyDeviceToDevice, e->stream));
+        from.from[k] = static_cast<char*>(e->buf[e->parity_host[c]]) + (size_t)c * bytes;
     }
     if (n_s > 0) {
-        int rc = bank_masses(e, n_s);
+        int rc = fill_bank(e, n_s, from);
         if (rc) return rc;
     }
     e->n_snaps_set = n_s;
@@ -1167,15 +1395,14 @@ int lbm_ensemble_set_snapshots_from_checkpoint(lbm_ensemble* e, int32_t n_s, con
     if (n_s < 0 || n_s > e->cfg.n_snapshots) return fail(LBM_ERR_ARG, "more snapshots than the bank holds");
     if (e->n_ckpt < 1 || k < 0 || k >= e->n_ckpt) return fail(LBM_ERR_ARG, "no such checkpoint");
     const size_t bytes = (size_t)e->clone_stride * e->elem_bytes;
+    SnapSources from{};
     for (int i = 0; i < n_s; ++i) {
         const int c = clones[i];
         if (c < 0 || c >= e->n) return fail(LBM_ERR_ARG, "clone index out of range");
-        LBM_CUDA(cudaMemcpyAsync(static_cast<char*>(e->snaps) + (size_t)i * bytes,
-                                 static_cast<char*>(e->ckpt) + ((size_t)c * e->n_ckpt + k) * bytes, bytes,
-                                 cudaMemcpyDeviceToDevice, e->stream));
+        from.from[i] = static_cast<char*>(e->ckpt) + ((size_t)c * e->n_ckpt + k) * bytes;
     }
     if (n_s > 0) {
-        int rc = bank_masses(e, n_s);
+        int rc = fill_bank(e, n_s, from);
         if (rc) return rc;
     }
     e->n_snaps_set = n_s;
@@ -1192,7 +1419,7 @@ int lbm_ensemble_clone(lbm_ensemble* e, const int32_t* parent_dev, double eps, u
         if (e->t_host[i] != t || e->parity_host[i] != e->parity_host[0])
             return fail(LBM_ERR_STATE, "cloning needs every clone at the same time");
     if (eps != 0.0) {
-        int rc = compute_masses(e, e->all_dev, e->n);
+        int rc = mass_partials(e, e->all_dev, e->n, parent_dev);
         if (rc) return rc;
     }
     int rc = run_perturb(e, parent_dev, -1, eps, seed, iter);
@@ -1226,10 +1453,9 @@ int lbm_ensemble_branch(lbm_ensemble* e, int32_t dst, int32_t src, int32_t t_b, 
     if (kc >= e->n_ckpt) return fail(LBM_ERR_ARG, "no checkpoint covers the branch time");
     const size_t bytes = (size_t)e->clone_stride * e->elem_bytes;
     char* ck = static_cast<char*>(e->ckpt);
-    // checkpoints 0..kc and the state at tc
-    for (int k = 0; k <= kc; ++k)
-        LBM_CUDA(cudaMemcpyAsync(ck + ((size_t)dst * e->n_ckpt + k) * bytes, ck + ((size_t)src * e->n_ckpt + k) * bytes,
-                                 bytes, cudaMemcpyDeviceToDevice, e->stream));
+    // checkpoints 0..kc (consecutive) and the state at tc
+    LBM_CUDA(cudaMemcpyAsync(ck + (size_t)dst * e->n_ckpt * bytes, ck + (size_t)src * e->n_ckpt * bytes,
+                             (kc + 1) * bytes, cudaMemcpyDeviceToDevice, e->stream));
     LBM_CUDA(cudaMemcpyAsync(static_cast<char*>(e->buf[e->parity_host[dst]]) + (size_t)dst * bytes,
                              ck + ((size_t)src * e->n_ckpt + kc) * bytes, bytes, cudaMemcpyDeviceToDevice, e->stream));
     if (e->cnn_score)  // the learned score of the shared checkpoints
@@ -1256,9 +1482,9 @@ int lbm_ensemble_branch(lbm_ensemble* e, int32_t dst, int32_t src, int32_t t_b, 
     }
     if (eps != 0.0) {
         LBM_CUDA(cudaMemcpyAsync(e->list_dev, &dst, sizeof(int32_t), cudaMemcpyHostToDevice, e->stream));
-        int rc = compute_masses(e, e->list_dev, 1);
+        int rc = mass_partials(e, e->list_dev, 1, nullptr);
         if (rc) return rc;
-        rc = run_perturb(e, e->all_dev, dst, eps, seed, iter);
+        rc = run_perturb(e, e->all_dev, dst, eps, seed, iter, e->list_dev, 1);
         if (rc) return rc;
         LBM_CUDA(cudaStreamSynchronize(e->stream));
     }
@@ -1278,7 +1504,7 @@ int lbm_ensemble_perturb(lbm_ensemble* e, int32_t n, const int32_t* clones, doub
     if (eps == 0.0) return LBM_OK;  // the identity
     if (e->n_snaps_set < 1) return fail(LBM_ERR_STATE, "perturbation needs the snapshot bank");
     LBM_CUDA(cudaMemcpyAsync(e->list_dev, clones, sizeof(int32_t) * n, cudaMemcpyHostToDevice, e->stream));
-    int rc = compute_masses(e, e->list_dev, n);
+    int rc = mass_partials(e, e->list_dev, n, nullptr);
     if (rc) return rc;
     rc = run_perturb(e, e->all_dev, kAllInPlace, eps, seed, iter, e->list_dev, n);
     if (rc) return rc;
@@ -1297,7 +1523,7 @@ int lbm_ensemble_set_perturbation(lbm_ensemble* e, int32_t mode)
 int lbm_ensemble_moments(lbm_ensemble* e, double* mass, double* px, double* py)
 {
     if (!e) return fail(LBM_ERR_ARG, "null ensemble");
-    int rc = compute_masses(e, e->all_dev, e->n);
+    int rc = compute_moments(e, e->all_dev, e->n);
     if (rc) return rc;
     std::vector<double> h(3 * (size_t)e->n);
     LBM_CUDA(cudaMemcpyAsync(h.data(), e->mass_dev, sizeof(double) * 3 * e->n, cudaMemcpyDeviceToHost, e->stream));
