@@ -1,8 +1,10 @@
 // Direct-sampling statistics of the drag (Sec. 3): the autocorrelation of the
 // drag fluctuations and its correlation time (caption of Fig. pdf_drag), and
 // the waiting-time return time r(a) of a level.  The ensemble's clones are
-// independent trajectories; their drag series over [t0, t1) are pooled.  FP64
-// throughout, every sum in a fixed order (results do not depend on timing).
+// independent trajectories; their drag series over [t0, t1) are pooled.  Means
+// and variances are FP64 sums in a fixed order, the products of the
+// autocorrelation exact integers (results do not depend on timing).
+#include <algorithm>
 #include <cmath>
 #include <limits>
 #include <vector>
@@ -28,72 +30,258 @@ __device__ double block_sum(double v, double* sh)
     return r;
 }
 
-// mean and variance of the pooled series (one block)
-__global__ void drag_moments_kernel(const double* drag, int32_t max_steps, int32_t n, int32_t t0, int32_t len,
-                                    double* mv)
+// The pooled series' moments, one block per clone: the sums; then, with the
+// mean of all, the sums of squares and the largest fluctuation (stat[0 .. n):
+// sums, [n .. 2n): squares, [2n .. 3n): largest |x|).  One block over the whole
+// series with a 64-bit division per element took 1356 us (64 x 6500).
+__global__ void drag_sum_kernel(const double* drag, int32_t max_steps, int32_t t0, int32_t len, double* stat)
 {
     __shared__ double sh[kStatThreads];
-    const int64_t total = (int64_t)n * len;
+    const double* row = drag + (int64_t)blockIdx.x * max_steps + t0;
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < total; i += kStatThreads) {
-        const int64_t c = i / len, t = i - c * len;
-        s += drag[c * max_steps + t0 + t];
-    }
-    const double mean = block_sum(s, sh) / (double)total;
-    double q = 0.0;
-    for (int64_t i = threadIdx.x; i < total; i += kStatThreads) {
-        const int64_t c = i / len, t = i - c * len;
-        const double x = drag[c * max_steps + t0 + t] - mean;
+    for (int t = threadIdx.x; t < len; t += kStatThreads) s += row[t];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) stat[blockIdx.x] = s;
+}
+
+// the sum of n values by a whole block, in a fixed order
+__device__ double sum_over(const double* v, int32_t n, double* sh)
+{
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += kStatThreads) s += v[i];
+    return block_sum(s, sh);
+}
+
+__global__ void drag_square_kernel(const double* drag, int32_t max_steps, int32_t n, int32_t t0, int32_t len,
+                                   double* stat)
+{
+    __shared__ double sh[kStatThreads];
+    const double mean = sum_over(stat, n, sh) / ((double)n * (double)len);
+    const double* row = drag + (int64_t)blockIdx.x * max_steps + t0;
+    double q = 0.0, top = 0.0;
+    for (int t = threadIdx.x; t < len; t += kStatThreads) {
+        const double x = row[t] - mean;
         q += x * x;
+        top = fmax(top, fabs(x));
     }
-    const double var = block_sum(q, sh) / (double)total;
+    q = block_sum(q, sh);
+    sh[threadIdx.x] = top;
+    __syncthreads();
+    for (int s = kStatThreads / 2; s > 0; s >>= 1) {
+        if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
-        mv[0] = mean;
-        mv[1] = var;
+        stat[n + blockIdx.x] = q;
+        stat[2 * n + blockIdx.x] = sh[0];
     }
 }
 
-// C(tau) for tau = blockIdx.x: mean over clones and t of x(t) x(t + tau) / var
-__global__ void autocorr_kernel(const double* drag, int32_t max_steps, int32_t n, int32_t t0, int32_t len,
-                                const double* mv, double* c)
+// The autocorrelation's products in fixed point.  FP64 runs at two products a
+// clock and SM on this GPU, 1.2 ms for the 7e8 products of 64 x 6500 steps and
+// 2000 lags; 32-bit integer multiply-adds with 64-bit sums run 32 times as many.
+// A fluctuation x is rounded to X = x 2^k with the largest below 2^54 (an error
+// of 2^-55 of the largest, below the 2^-53 of an FP64 fluctuation) and split
+// into X = hi 2^28 + lo, |hi| <= 2^26 + 1, |lo| <= 2^27.  Every product and every
+// sum after that is exact, so the result does not depend on their order.
+constexpr int kLimb = 28;
+
+// k of the quantisation; 0 for an all-zero or a non-finite series
+__device__ int fixed_exponent(const double* stat, int32_t n, double* sh)
+{
+    double top = 0.0;
+    for (int i = threadIdx.x; i < n; i += kStatThreads) top = fmax(top, stat[2 * n + i]);
+    sh[threadIdx.x] = top;
+    __syncthreads();
+    for (int s = kStatThreads / 2; s > 0; s >>= 1) {
+        if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
+        __syncthreads();
+    }
+    top = sh[0];
+    __syncthreads();
+    return top > 0.0 && isfinite(top) ? 53 - ilogb(top) : 0;
+}
+
+// the limbs of every clone's fluctuations, [n][pitch] each, zeros past the series
+__global__ void drag_limbs_kernel(const double* drag, int32_t max_steps, int32_t n, int32_t t0, int32_t len,
+                                  const double* stat, int32_t pitch, int32_t* hi, int32_t* lo)
 {
     __shared__ double sh[kStatThreads];
-    const int tau = blockIdx.x;
-    const int m = len - tau;
-    const double mean = mv[0];
-    const int64_t total = (int64_t)n * m;
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < total; i += kStatThreads) {
-        const int64_t cl = i / m, t = i - cl * m;
-        const double* row = drag + cl * max_steps + t0;
-        s += (row[t] - mean) * (row[t + tau] - mean);
+    const double mean = sum_over(stat, n, sh) / ((double)n * (double)len);
+    const int k = fixed_exponent(stat, n, sh);
+    const double s1 = scalbn(1.0, k / 2), s2 = scalbn(1.0, k - k / 2);
+    const int64_t c = blockIdx.y;
+    const int t = blockIdx.x * kStatThreads + threadIdx.x;
+    if (t >= pitch) return;
+    long long X = 0;
+    if (t < len) X = __double2ll_rn((drag[c * max_steps + t0 + t] - mean) * s1 * s2);
+    const long long h = (X + (1ll << (kLimb - 1))) >> kLimb;
+    hi[c * pitch + t] = (int32_t)h;
+    lo[c * pitch + t] = (int32_t)(X - (h << kLimb));
+}
+
+// Exact sums of products X(t) X(t + lag): a thread owns four consecutive lags
+// and takes four times t at once from registers (16 products, 48 multiply-adds,
+// for six 16-byte shared-memory loads; three multiply-adds a product instead of
+// four through (hi + lo)(hi' + lo') - hi hi' - lo lo').  A block takes kCorrLags lags and walks
+// its share of the (clone, kCorrTime steps) tasks; partial[split][lag].
+constexpr int kCorrThreads = 128, kCorrLags = 4 * kCorrThreads, kCorrTime = 512, kCorrFlush = 128;
+
+__global__ void __launch_bounds__(kCorrThreads) autocorr_kernel(const int32_t* hi, const int32_t* lo, int32_t n,
+                                                                int32_t len, int32_t pitch, int32_t n_lags,
+                                                                __int128* partial)
+{
+    constexpr int kWin = kCorrTime + kCorrLags + 4;
+    __shared__ __align__(16) int32_t ah[kCorrTime], al[kCorrTime], as[kCorrTime], bh[kWin], bl[kWin], bs[kWin];
+    const int chunks = (len + kCorrTime - 1) / kCorrTime, tasks = n * chunks;
+    const int lag0 = blockIdx.x * kCorrLags, l0 = 4 * threadIdx.x;
+    __int128 sum[4] = {0, 0, 0, 0};
+    for (int task = blockIdx.y; task < tasks; task += gridDim.y) {
+        const int c = task / chunks, tb = (task - c * chunks) * kCorrTime;
+        if (tb + lag0 >= len) continue;  // block-uniform: every product is past the series
+        const int32_t *rh = hi + (int64_t)c * pitch, *rl = lo + (int64_t)c * pitch;
+        __syncthreads();
+        for (int i = threadIdx.x; i < kCorrTime; i += kCorrThreads) {
+            ah[i] = rh[tb + i];  // the rows are zero up to their pitch
+            al[i] = rl[tb + i];
+            as[i] = ah[i] + al[i];
+        }
+        for (int i = threadIdx.x; i < kWin; i += kCorrThreads) {
+            const int t = tb + lag0 + i;
+            bh[i] = t < pitch ? rh[t] : 0;
+            bl[i] = t < pitch ? rl[t] : 0;
+            bs[i] = bh[i] + bl[i];
+        }
+        __syncthreads();
+        for (int f = 0; f < kCorrTime; f += kCorrFlush) {
+            // 128 products of each kind: below 2^60, 2^62 and 2^63
+            long long hh[4] = {0, 0, 0, 0}, ll[4] = {0, 0, 0, 0}, ss[4] = {0, 0, 0, 0};
+            auto at = [](const int32_t* v) { return *reinterpret_cast<const int4*>(v); };
+            int4 wh = at(bh + f + l0), wl = at(bl + f + l0), ws = at(bs + f + l0);
+#pragma unroll 2
+            for (int t = f; t < f + kCorrFlush; t += 4) {
+                const int4 vh = at(bh + t + 4 + l0), vl = at(bl + t + 4 + l0), vs = at(bs + t + 4 + l0);
+                auto products = [](long long (&acc)[4], const int4& x, const int4& w, const int4& v) {
+                    const int X[4] = {x.x, x.y, x.z, x.w}, Y[8] = {w.x, w.y, w.z, w.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int d = 0; d < 4; ++d)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc[j] += (long long)X[d] * Y[d + j];
+                };
+                products(hh, at(ah + t), wh, vh);
+                products(ll, at(al + t), wl, vl);
+                products(ss, at(as + t), ws, vs);
+                wh = vh;
+                wl = vl;
+                ws = vs;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                sum[j] += ((__int128)hh[j] << (2 * kLimb)) + (((__int128)ss[j] - hh[j] - ll[j]) << kLimb) + (__int128)ll[j];
+        }
     }
-    const double sum = block_sum(s, sh);
-    if (threadIdx.x == 0) c[tau] = sum / (double)total / mv[1];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (lag0 + l0 + j < n_lags) partial[(int64_t)blockIdx.y * n_lags + lag0 + l0 + j] = sum[j];
+}
+
+// C(lag) = sum of products / their number / variance; the first lag with C <= 0.
+// A block takes 32 lags, each of its warps a part of the splits.
+__global__ void __launch_bounds__(kStatThreads) autocorr_final_kernel(const __int128* partial, int32_t splits, int32_t n_lags, const double* stat,
+                                      int32_t n, int32_t len, double* c, int32_t* first)
+{
+    __shared__ double sh[kStatThreads];
+    const double var = sum_over(stat + n, n, sh) / ((double)n * (double)len);
+    const int k = fixed_exponent(stat, n, sh);
+    __shared__ __int128 part[kStatThreads / 32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lag = blockIdx.x * 32 + lane;
+    __int128 s = 0;
+    if (lag < n_lags)
+        for (int i = warp; i < splits; i += kStatThreads / 32) s += partial[(int64_t)i * n_lags + lag];
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || lag >= n_lags) return;
+    for (int w = 1; w < kStatThreads / 32; ++w) s += part[w][lane];
+    const double x = scalbn(scalbn((double)(long long)(s >> 64) * 0x1.0p64 + (double)(unsigned long long)s, -k), -k);
+    const double v = x / ((double)n * (double)(len - lag)) / var;
+    c[lag] = v;
+    if (v <= 0.0) atomicMin(first, lag);
 }
 
 // events of level j in clone c: up-crossings to >= a, merged with an earlier
-// one when the series was >= a within the last `gap` steps
-__global__ void upcross_kernel(const double* drag, int32_t max_steps, int32_t n, int32_t t0, int32_t len,
-                               const double* levels, int32_t n_levels, int32_t gap, long long* ev)
+// one when the series was >= a within the last `gap` steps.  So step t >= 1 is
+// an event if the series is >= a there and no step in the max(gap, 1) before it
+// is.  A block per (clone, level), a warp per segment of the series, 32 steps a
+// time by ballots (one thread per series took 1108 us, 64 x 6500); the first
+// step >= a of each segment is judged against the segments before it at the end.
+constexpr int kUpWarps = 8;
+
+__global__ void __launch_bounds__(32 * kUpWarps) upcross_kernel(const double* drag, int32_t max_steps, int32_t t0,
+                                                                int32_t len, const double* levels, int32_t gap,
+                                                                unsigned long long* ev)
 {
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= n * n_levels) return;
-    const int j = id / n, c = id - j * n;
-    const double a = levels[j];
-    const double* row = drag + (int64_t)c * max_steps + t0;
-    long long count = 0;
-    int last_above = -1;
-    bool above_prev = false;
-    for (int t = 0; t < len; ++t) {
-        const bool above = row[t] >= a;
-        if (above) {
-            if (t > 0 && !above_prev && (last_above < 0 || t - last_above > gap)) ++count;
-            last_above = t;
-        }
-        above_prev = above;
+    __shared__ int count[kUpWarps], first[kUpWarps], last[kUpWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quiet = max(gap, 1);
+    const double a = levels[blockIdx.y];
+    const double* row = drag + (int64_t)blockIdx.x * max_steps + t0;
+    const int seg = ((len + kUpWarps - 1) / kUpWarps + 31) & ~31, b = min(warp * seg, len), e = min(b + seg, len);
+    int n_ev = 0, head = -1, before = -1;  // before: the last step >= a so far
+    for (int t = b; t < e; t += 32) {
+        const bool up = t + lane < e && row[t + lane] >= a;
+        const uint32_t m = __ballot_sync(0xffffffffu, up);
+        if (m == 0u) continue;
+        if (head < 0) head = t + __ffs(m) - 1;
+        const uint32_t lower = m & ((1u << lane) - 1u);
+        const int prev = lower ? t + 31 - __clz(lower) : before;
+        n_ev += __popc(__ballot_sync(0xffffffffu, up && prev >= 0 && t + lane - prev > quiet));
+        before = t + 31 - __clz(m);
     }
-    ev[id] = count;
+    if (lane == 0) {
+        count[warp] = n_ev;
+        first[warp] = head;
+        last[warp] = before;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long total = 0;
+        int prev = -1;
+        for (int w = 0; w < kUpWarps; ++w) {
+            if (first[w] < 0) continue;
+            total += count[w] + (first[w] > 0 && (prev < 0 || first[w] - prev > quiet) ? 1 : 0);
+            prev = last[w];
+        }
+        if (total) atomicAdd(ev + blockIdx.y, total);
+    }
+}
+
+// A workspace of at least `bytes` for one call: the ensemble's own, grown on
+// demand and kept until the ensemble is destroyed (used in its stream's order),
+// or, where it would have to grow while the stream is being captured, an
+// allocation of the captured work itself (temporary: released by the caller).
+struct Workspace {
+    char* p = nullptr;
+    bool temporary = false;
+};
+
+int stat_workspace(lbm_ensemble* e, size_t bytes, Workspace* ws)
+{
+    if (e->stat_bytes < bytes) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        LBM_CUDA(cudaStreamIsCapturing(e->stream, &capturing));
+        if (capturing != cudaStreamCaptureStatusNone) {
+            LBM_CUDA(cudaMallocAsync((void**)&ws->p, bytes, e->stream));
+            ws->temporary = true;
+            return LBM_OK;
+        }
+        LBM_CUDA(cudaStreamSynchronize(e->stream));
+        if (e->stat_ws) cudaFree(e->stat_ws);
+        e->stat_ws = nullptr;
+        e->stat_bytes = 0;
+        LBM_CUDA(cudaMalloc(&e->stat_ws, bytes));
+        e->stat_bytes = bytes;
+    }
+    ws->p = static_cast<char*>(e->stat_ws);
+    return LBM_OK;
 }
 
 int check_window(lbm_ensemble* e, int32_t t0, int32_t t1)
@@ -116,23 +304,37 @@ int lbm_drag_autocorrelation(lbm_ensemble* e, int32_t t0, int32_t t1, int32_t ma
     if (!e || !c_dev) return fail(LBM_ERR_ARG, "lbm_drag_autocorrelation: null argument");
     if (int rc = check_window(e, t0, t1)) return rc;
     if (max_lag < 0 || max_lag >= t1 - t0) return fail(LBM_ERR_ARG, "lbm_drag_autocorrelation: need 0 <= max_lag < t1 - t0");
-    double* mv = e->mass_dev;  // [N] x 3 doubles of scratch: two are enough
-    drag_moments_kernel<<<1, kStatThreads, 0, e->stream>>>(e->drag, e->cfg.max_steps, e->n, t0, t1 - t0, mv);
-    autocorr_kernel<<<max_lag + 1, kStatThreads, 0, e->stream>>>(e->drag, e->cfg.max_steps, e->n, t0, t1 - t0, mv,
-                                                                  c_dev);
+    // workspace: moments of each clone, the limbs of the fluctuations (rows padded
+    // so that a task's loads stay in its row), exact partial sums per split
+    const int32_t len = t1 - t0, n = e->n, lags = max_lag + 1, pitch = (len + kCorrTime - 1) / kCorrTime * kCorrTime;
+    const int lag_tiles = (lags + kCorrLags - 1) / kCorrLags;
+    const int64_t tasks = (int64_t)n * (pitch / kCorrTime);
+    if (tasks > INT32_MAX) return fail(LBM_ERR_ARG, "lbm_drag_autocorrelation: series too long");
+    const int splits = (int)std::min<int64_t>(tasks, std::max(1, 152 * 12 / lag_tiles));
+    const size_t limb_bytes = sizeof(int32_t) * (size_t)n * pitch, stat_bytes = (sizeof(double) * 3 * n + 15) / 16 * 16;
+    Workspace ws;
+    if (int rc = stat_workspace(e, 16 + sizeof(__int128) * (size_t)splits * lags + stat_bytes + 2 * limb_bytes, &ws)) return rc;
+    int32_t* first = reinterpret_cast<int32_t*>(ws.p);
+    __int128* partial = reinterpret_cast<__int128*>(ws.p + 16);
+    double* stat = reinterpret_cast<double*>(ws.p + 16 + sizeof(__int128) * (size_t)splits * lags);
+    int32_t* hi = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(stat) + stat_bytes);
+    int32_t* lo = hi + (size_t)n * pitch;
+    LBM_CUDA(cudaMemsetAsync(first, 0x7f, sizeof(int32_t), e->stream));
+    drag_sum_kernel<<<n, kStatThreads, 0, e->stream>>>(e->drag, e->cfg.max_steps, t0, len, stat);
+    drag_square_kernel<<<n, kStatThreads, 0, e->stream>>>(e->drag, e->cfg.max_steps, n, t0, len, stat);
+    drag_limbs_kernel<<<dim3((pitch + kStatThreads - 1) / kStatThreads, n), kStatThreads, 0, e->stream>>>(
+        e->drag, e->cfg.max_steps, n, t0, len, stat, pitch, hi, lo);
+    autocorr_kernel<<<dim3(lag_tiles, splits), kCorrThreads, 0, e->stream>>>(hi, lo, n, len, pitch, lags, partial);
+    autocorr_final_kernel<<<(lags + 31) / 32, kStatThreads, 0, e->stream>>>(
+        partial, splits, lags, stat, n, len, c_dev, first);
     LBM_CUDA(cudaGetLastError());
-    count_launches(2);
+    count_launches(5);
     if (tau_c) {
-        std::vector<double> c(max_lag + 1);
-        LBM_CUDA(cudaMemcpyAsync(c.data(), c_dev, sizeof(double) * c.size(), cudaMemcpyDeviceToHost, e->stream));
+        LBM_CUDA(cudaMemcpyAsync(tau_c, first, sizeof(int32_t), cudaMemcpyDeviceToHost, e->stream));
         LBM_CUDA(cudaStreamSynchronize(e->stream));
-        *tau_c = -1;
-        for (int i = 0; i <= max_lag; ++i)
-            if (c[i] <= 0.0) {
-                *tau_c = i;
-                break;
-            }
+        if (*tau_c > max_lag) *tau_c = -1;
     }
+    if (ws.temporary) LBM_CUDA(cudaFreeAsync(ws.p, e->stream));
     return LBM_OK;
 }
 
@@ -142,25 +344,19 @@ int lbm_drag_return_times(lbm_ensemble* e, int32_t t0, int32_t t1, int32_t n_lev
     if (!e || !levels_dev || !events || !r) return fail(LBM_ERR_ARG, "lbm_drag_return_times: null argument");
     if (int rc = check_window(e, t0, t1)) return rc;
     if (n_levels < 1 || n_levels > 4096 || gap < 0) return fail(LBM_ERR_ARG, "lbm_drag_return_times: levels or gap");
-    const int64_t m = (int64_t)e->n * n_levels;
-    long long* ev = nullptr;
-    LBM_CUDA(cudaMallocAsync((void**)&ev, sizeof(long long) * m, e->stream));
-    upcross_kernel<<<(int)((m + 127) / 128), 128, 0, e->stream>>>(e->drag, e->cfg.max_steps, e->n, t0, t1 - t0,
-                                                                   levels_dev, n_levels, gap, ev);
-    cudaError_t err = cudaGetLastError();
-    std::vector<long long> h(m);
-    if (err == cudaSuccess)
-        err = cudaMemcpyAsync(h.data(), ev, sizeof(long long) * m, cudaMemcpyDeviceToHost, e->stream);
-    cudaFreeAsync(ev, e->stream);
-    if (err == cudaSuccess) err = cudaStreamSynchronize(e->stream);
-    if (err != cudaSuccess) return cuda_fail(err, "lbm_drag_return_times");
+    Workspace ws;
+    if (int rc = stat_workspace(e, sizeof(unsigned long long) * n_levels, &ws)) return rc;
+    auto* ev = reinterpret_cast<unsigned long long*>(ws.p);
+    LBM_CUDA(cudaMemsetAsync(ev, 0, sizeof(unsigned long long) * n_levels, e->stream));
+    upcross_kernel<<<dim3(e->n, n_levels), 32 * kUpWarps, 0, e->stream>>>(e->drag, e->cfg.max_steps, t0, t1 - t0,
+                                                                          levels_dev, gap, ev);
+    LBM_CUDA(cudaGetLastError());
     count_launches(1);
+    LBM_CUDA(cudaMemcpyAsync(events, ev, sizeof(int64_t) * n_levels, cudaMemcpyDeviceToHost, e->stream));
+    LBM_CUDA(cudaStreamSynchronize(e->stream));
     const double observed = (double)e->n * (double)(t1 - t0);
     for (int j = 0; j < n_levels; ++j) {
-        long long s = 0;
-        for (int c = 0; c < e->n; ++c) s += h[(int64_t)j * e->n + c];
-        events[j] = s;
-        r[j] = s > 0 ? observed / (double)s : std::numeric_limits<double>::infinity();
+        r[j] = events[j] > 0 ? observed / (double)events[j] : std::numeric_limits<double>::infinity();
     }
     return LBM_OK;
 }
