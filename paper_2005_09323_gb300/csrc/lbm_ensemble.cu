@@ -865,15 +865,32 @@ int launch_chunk(lbm_ensemble* e, int vi, const int32_t* list_dev, int n_list, i
     if (!hit) {
         if (!e->cap_stream) LBM_CUDA(cudaStreamCreateWithFlags(&e->cap_stream, cudaStreamNonBlocking));
         LBM_CUDA(cudaStreamBeginCapture(e->cap_stream, cudaStreamCaptureModeRelaxed));
+        // observables run beside the next step, which reads the same state; the
+        // step after that overwrites it and waits for them
+        cudaStream_t side = nullptr;
+        cudaEvent_t stepped = nullptr, seen[2] = {nullptr, nullptr};
         cudaError_t launch_err = cudaSuccess;
+        auto ok = [&](cudaError_t err) { return (launch_err = err) == cudaSuccess; };
+        if (e->observe && ok(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking)) &&
+            ok(cudaEventCreateWithFlags(&stepped, cudaEventDisableTiming)) &&
+            ok(cudaEventCreateWithFlags(&seen[0], cudaEventDisableTiming)))
+            ok(cudaEventCreateWithFlags(&seen[1], cudaEventDisableTiming));
         for (size_t i = 0; i < first.size() && launch_err == cudaSuccess; ++i) {
-            launch_err = launch(params(i), e->cap_stream);
-            if (launch_err == cudaSuccess && e->observe &&
-                observables_launch(e, list_dev, n_list, first[i], e->cap_stream))
+            if (e->observe && i >= 2 && !ok(cudaStreamWaitEvent(e->cap_stream, seen[i & 1], 0))) break;
+            if (!ok(launch(params(i), e->cap_stream)) || !e->observe) continue;
+            if (!ok(cudaEventRecord(stepped, e->cap_stream)) || !ok(cudaStreamWaitEvent(side, stepped, 0))) break;
+            if (observables_launch(e, list_dev, n_list, first[i], side))
                 launch_err = cudaGetLastError();
+            else
+                ok(cudaEventRecord(seen[i & 1], side));
         }
+        for (size_t k = 0; k < std::min<size_t>(first.size(), 2); ++k)
+            if (e->observe && launch_err == cudaSuccess) ok(cudaStreamWaitEvent(e->cap_stream, seen[k], 0));
         cudaGraph_t graph = nullptr;
         const cudaError_t end_err = cudaStreamEndCapture(e->cap_stream, &graph);
+        for (cudaEvent_t ev : {stepped, seen[0], seen[1]})
+            if (ev) cudaEventDestroy(ev);
+        if (side) cudaStreamDestroy(side);
         if (launch_err != cudaSuccess || end_err != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
             cudaGetLastError();

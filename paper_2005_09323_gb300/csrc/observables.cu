@@ -21,17 +21,22 @@ namespace {
 
 constexpr int kObsThreads = 128;
 
-__device__ double obs_block_sum(double v, double* sh)
+// sum of v[0 .. count) for the four quantities, one warp each: strided partial
+// sums over kObsThreads, then a tree over them, in the order of a block-wide
+// tree (the lanes hold entries l, l + 32, l + 64, l + 96 of it)
+template <typename F>
+__device__ double obs_warp_sum(int count, F&& v)
 {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = kObsThreads / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    double a[kObsThreads / 32];
+#pragma unroll
+    for (int k = 0; k < kObsThreads / 32; ++k) {
+        a[k] = 0.0;
+        for (int i = (threadIdx.x & 31) + 32 * k; i < count; i += kObsThreads) a[k] += v(i);
     }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+    double s = (a[0] + a[2]) + (a[1] + a[3]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    return s;
 }
 
 // density and velocity of node (x, y) of a post-collision state
@@ -51,45 +56,51 @@ __device__ void node_macro(const typename Codec<S>::T* st, int64_t plane, int32_
     ux = (jx - hgx) / rho;
 }
 
+// One block per clone.  Latency bounds it: 96 nodes of a 16 x 16 square, FP64
+// arithmetic at two operations a clock and SM.  With the nodes spread over the
+// threads and one warp per sum it takes a fraction of the 16 us of a block that
+// gave each of 16 threads six nodes in turn.
 template <int S>
 __global__ void __launch_bounds__(kObsThreads)
 observables_kernel(const void* buf0, const void* buf1, const int32_t* parity, const int32_t* list, int32_t step,
                    int64_t clone_stride, int64_t plane, int32_t pitch, int32_t ox0, int32_t ox1, int32_t oy0,
-                   int32_t oy1, double hgx, float inv_scale, const int32_t* t, double* obs, int32_t max_steps)
+                   int32_t oy1, double hgx, float inv_scale, const int32_t* t, double* obs, int32_t max_steps, bool staged)
 {
     using T = typename Codec<S>::T;
-    __shared__ double sh[kObsThreads];
+    // the nodes the observables need, one per thread: the columns before and
+    // after the square (densities), then four rows of its width (velocities):
+    // above it at distances 1/2 and 3/2, below it at 1/2 and 3/2
+    extern __shared__ double node[];
     const int c = list[blockIdx.x];
     const int cur = parity[c] ^ (step & 1);
     const T* st = static_cast<const T*>(cur ? buf0 : buf1) + (int64_t)c * clone_stride;  // this step's state
     constexpr double kCs2 = 1.0 / 3.0;
-    double pfb = 0.0, pbase = 0.0, gt = 0.0, gb = 0.0;
-    double rho, u1, u2;
-    for (int y = oy0 + threadIdx.x; y < oy1; y += kObsThreads) {
-        node_macro<S>(st, plane, pitch, ox0 - 1, y, inv_scale, hgx, rho, u1);
-        pfb += kCs2 * rho;
-        node_macro<S>(st, plane, pitch, ox1, y, inv_scale, hgx, rho, u1);
-        pbase += kCs2 * rho;
-    }
-    for (int x = ox0 + threadIdx.x; x < ox1; x += kObsThreads) {
-        node_macro<S>(st, plane, pitch, x, oy1, inv_scale, hgx, rho, u1);
-        node_macro<S>(st, plane, pitch, x, oy1 + 1, inv_scale, hgx, rho, u2);
-        gt += (9.0 * u1 - u2) / 3.0;
-        node_macro<S>(st, plane, pitch, x, oy0 - 1, inv_scale, hgx, rho, u1);
-        node_macro<S>(st, plane, pitch, x, oy0 - 2, inv_scale, hgx, rho, u2);
-        gb -= (9.0 * u1 - u2) / 3.0;
-    }
-    pfb = obs_block_sum(pfb, sh);
-    pbase = obs_block_sum(pbase, sh);
-    gt = obs_block_sum(gt, sh);
-    gb = obs_block_sum(gb, sh);
-    if (threadIdx.x == 0) {
-        double* o = obs + ((int64_t)c * max_steps + t[c] + step) * 4;
-        o[0] = pfb;
-        o[1] = pbase;
-        o[2] = gt / (ox1 - ox0);
-        o[3] = gb / (ox1 - ox0);
-    }
+    const int h = oy1 - oy0, w = ox1 - ox0;
+    auto value = [&](int i) {
+        double rho, ux;
+        if (i < 2 * h) {
+            node_macro<S>(st, plane, pitch, i < h ? ox0 - 1 : ox1, oy0 + (i < h ? i : i - h), inv_scale, hgx, rho, ux);
+            return rho;
+        }
+        const int k = (i - 2 * h) / w, x = ox0 + (i - 2 * h - k * w);
+        const int y = k == 0 ? oy1 : (k == 1 ? oy1 + 1 : (k == 2 ? oy0 - 1 : oy0 - 2));
+        node_macro<S>(st, plane, pitch, x, y, inv_scale, hgx, rho, ux);
+        return ux;
+    };
+    if (staged)
+        for (int i = threadIdx.x; i < 2 * h + 4 * w; i += kObsThreads) node[i] = value(i);
+    __syncthreads();
+    auto at = [&](int i) { return staged ? node[i] : value(i); };
+    auto u = [&](int i) { return at(2 * h + i); };
+    const int warp = threadIdx.x >> 5;
+    double v;
+    if (warp < 2)
+        v = obs_warp_sum(h, [&](int i) { return kCs2 * at(warp * h + i); });
+    else if (warp == 2)
+        v = obs_warp_sum(w, [&](int i) { return (9.0 * u(i) - u(w + i)) / 3.0; });
+    else
+        v = obs_warp_sum(w, [&](int i) { return -((9.0 * u(2 * w + i) - u(3 * w + i)) / 3.0); });
+    if ((threadIdx.x & 31) == 0) obs[((int64_t)c * max_steps + t[c] + step) * 4 + warp] = warp < 2 ? v : v / w;
 }
 
 }  // namespace
@@ -99,24 +110,28 @@ int observables_launch(lbm_ensemble* e, const int32_t* list_dev, int32_t n_list,
     const lbm_config& c = e->cfg;
     const int ox0 = c.obs_x0, ox1 = c.obs_x0 + c.obs_w, oy0 = c.obs_y0, oy1 = c.obs_y0 + c.obs_h;
     const double hgx = 0.5 * c.gx;
+    // a square whose nodes do not fit 48 KB is evaluated without staging them
+    const size_t nodes = sizeof(double) * (2 * (size_t)c.obs_h + 4 * (size_t)c.obs_w);
+    const bool staged = nodes <= 48 * 1024;
+    const size_t smem = staged ? nodes : 0;
     switch (c.storage) {
     case kFP32:
-        observables_kernel<kFP32><<<n_list, kObsThreads, 0, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
+        observables_kernel<kFP32><<<n_list, kObsThreads, smem, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
                                                                  e->clone_stride, e->plane, e->pitch, ox0, ox1, oy0,
                                                                  oy1, hgx, e->inv_scale, e->t_dev, e->obs,
-                                                                 c.max_steps);
+                                                                 c.max_steps, staged);
         break;
     case kFP16:
-        observables_kernel<kFP16><<<n_list, kObsThreads, 0, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
+        observables_kernel<kFP16><<<n_list, kObsThreads, smem, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
                                                                  e->clone_stride, e->plane, e->pitch, ox0, ox1, oy0,
                                                                  oy1, hgx, e->inv_scale, e->t_dev, e->obs,
-                                                                 c.max_steps);
+                                                                 c.max_steps, staged);
         break;
     default:
-        observables_kernel<kBF16><<<n_list, kObsThreads, 0, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
+        observables_kernel<kBF16><<<n_list, kObsThreads, smem, s>>>(e->buf[0], e->buf[1], e->parity_dev, list_dev, step,
                                                                  e->clone_stride, e->plane, e->pitch, ox0, ox1, oy0,
                                                                  oy1, hgx, e->inv_scale, e->t_dev, e->obs,
-                                                                 c.max_steps);
+                                                                 c.max_steps, staged);
     }
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
