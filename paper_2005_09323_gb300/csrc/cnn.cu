@@ -344,7 +344,10 @@ __global__ void __launch_bounds__(128, 8) input_conv_kernel(const bf16* __restri
     }
 }
 
-// dW partials: block-persistent over output tiles; D[co][k] += dY^T patch
+// dW partials: block-persistent over output tiles; D[co][k] += dY^T patch.  The
+// next tile's halo and output gradient are fetched with cp.async while the
+// current tile is multiplied (the input layer's kernel took 158 us loading
+// each tile between two barriers, 64 x 256 and batch 256).
 template <int CIN>
 __global__ void __launch_bounds__(128) conv_wgrad_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dy,
                                                          int B, int H, int W, float* __restrict__ partial)
@@ -353,8 +356,9 @@ __global__ void __launch_bounds__(128) conv_wgrad_kernel(const bf16* __restrict_
     constexpr int NT = KP / 8;           // feature tiles of 8
     constexpr int NTW = (NT + 3) / 4;    // per warp
     constexpr int REAL_NT = 9 * CIN / 8; // tiles of real taps; the next one holds the bias column
-    __shared__ __align__(16) bf16 s_in[kHPix * CIN];
-    __shared__ __align__(16) bf16 s_dy[kTH * kTW * kC];
+    constexpr int NBUF = CIN == kCin0 ? 2 : 1;  // the 32-channel tiles would not fit 48 KB twice
+    __shared__ __align__(16) bf16 s_in2[NBUF][kHPix * CIN];
+    __shared__ __align__(16) bf16 s_dy2[NBUF][kTH * kTW * kC];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     float acc[2][NTW][4];
@@ -366,19 +370,41 @@ __global__ void __launch_bounds__(128) conv_wgrad_kernel(const bf16* __restrict_
             for (int r = 0; r < 4; ++r) acc[m][n][r] = 0.f;
     const int tiles_x = W / kTW, tiles_y = H / kTH;
     const int total = B * tiles_x * tiles_y;
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    auto fetch = [&](int tile, int buf) {
         const int b = tile / (tiles_x * tiles_y);
         const int rem = tile - b * tiles_x * tiles_y;
-        const int ty0 = (rem / tiles_x) * kTH, tx0 = (rem % tiles_x) * kTW;
-        __syncthreads();
-        load_halo<CIN>(s_in, x, b, ty0, tx0, H, W);
-        for (int i = threadIdx.x; i < kTH * kTW * 4; i += blockDim.x) {
+        const int ty0 = (rem / tiles_x) * kTH, tx0 = (rem - (rem / tiles_x) * tiles_x) * kTW;
+        constexpr int CH = CIN / 8;
+        for (int i = threadIdx.x; i < kHPix * CH; i += 128) {
+            const int pix = i / CH, ch = i - pix * CH;
+            const int hr = pix / kHW, hc = pix - hr * kHW;
+            const int gy = ty0 + hr - 1, gx = tx0 + hc - 1;
+            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;  // zeros outside the image
+            const bf16* src = in ? x + (((int64_t)b * H + gy) * W + gx) * CIN + ch * 8 : x;
+            cp_async16(s_in2[buf] + halo_off<CIN>(pix, ch), src, in ? 16u : 0u);
+        }
+        for (int i = threadIdx.x; i < kTH * kTW * 4; i += 128) {
             const int pix = i >> 2, ch = i & 3;
             const int gy = ty0 + pix / kTW, gx = tx0 + (pix % kTW);
-            *reinterpret_cast<uint4*>(s_dy + halo_off<32>(pix, ch)) =
-                *reinterpret_cast<const uint4*>(dy + (((int64_t)b * H + gy) * W + gx) * kC + ch * 8);
+            cp_async16(s_dy2[buf] + halo_off<32>(pix, ch), dy + (((int64_t)b * H + gy) * W + gx) * kC + ch * 8, 16u);
+        }
+        cp_async_commit();
+    };
+    if (NBUF == 2 && (int)blockIdx.x < total) fetch(blockIdx.x, 0);
+    for (int tile = blockIdx.x, k = 0; tile < total; tile += gridDim.x, ++k) {
+        const int buf = NBUF == 2 ? k & 1 : 0;
+        __syncthreads();  // the buffer to be filled is read out
+        if (NBUF == 1) {
+            fetch(tile, 0);
+            cp_async_wait<0>();
+        } else if (tile + (int)gridDim.x < total) {
+            fetch(tile + gridDim.x, buf ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
         }
         __syncthreads();
+        const bf16 *s_in = s_in2[buf], *s_dy = s_dy2[buf];
 #pragma unroll 1
         for (int r = 0; r < kTH; ++r) {
             // A = dY^T (co x 16 pixels of tile row r) via transposed ldmatrix
@@ -434,48 +460,69 @@ __global__ void __launch_bounds__(128) conv_wgrad_kernel(const bf16* __restrict_
         }
 }
 
-__global__ void reduce_partials_kernel(const float* partial, int nblk, int n, float* out)
+// out[i] = partial[0][i] + partial[1][i] + ... in that order.  A block takes 32
+// columns: its warps bring a batch of rows to shared memory at once and the
+// first one adds them up (one thread per column waiting for each load took
+// 80 us for the input layer's 1216 partials).
+constexpr int kReduceRows = 256;
+
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const float* partial, int nblk, int n, float* out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    __shared__ float rows[kReduceRows][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += partial[(int64_t)b * n + i];
-    out[i] = s;
+    for (int b0 = 0; b0 < nblk; b0 += kReduceRows) {
+        const int nb = min(kReduceRows, nblk - b0);
+#pragma unroll 8
+        for (int b = warp; b < nb; b += 8) rows[b][lane] = i < n ? partial[(int64_t)(b0 + b) * n + i] : 0.f;
+        __syncthreads();
+        if (warp == 0)
+#pragma unroll 8
+            for (int b = 0; b < nb; ++b) s += rows[b][lane];
+        __syncthreads();
+    }
+    if (warp == 0 && i < n) out[i] = s;
 }
 
-// global mean pool over the pixels of the last activation, then the linear head
-__global__ void head_forward_kernel(const bf16* __restrict__ act, int P, const float* __restrict__ head,
-                                   float* __restrict__ pooled, float* __restrict__ pred)
+// global mean pool over the pixels of the last activation, then the linear head.
+// Four threads share a pixel (16 bytes, 8 channels each), so a warp reads 512
+// consecutive bytes; 1024 threads keep enough loads in flight for one block per
+// sample (with 256 threads of a whole pixel each: 58 us for 64 samples of 64 x
+// 256, 65 us for 256).
+constexpr int kHeadThreads = 1024;
+
+__global__ void __launch_bounds__(kHeadThreads) head_forward_kernel(const bf16* __restrict__ act, int P,
+                                                                    const float* __restrict__ head,
+                                                                    float* __restrict__ pooled,
+                                                                    float* __restrict__ pred)
 {
     __shared__ float sh[256][kC + 1];
-    const int b = blockIdx.x;
-    float s[kC];
+    const int b = blockIdx.x, row = threadIdx.x >> 2, c0 = (threadIdx.x & 3) * 8;
+    float s[8];
 #pragma unroll
-    for (int c = 0; c < kC; ++c) s[c] = 0.f;
-    for (int p = threadIdx.x; p < P; p += 256) {
-        const uint4* src = reinterpret_cast<const uint4*>(act + ((int64_t)b * P + p) * kC);
+    for (int c = 0; c < 8; ++c) s[c] = 0.f;
+    const uint4* src = reinterpret_cast<const uint4*>(act + (int64_t)b * P * kC) + (threadIdx.x & 3);
+#pragma unroll 8
+    for (int p = row; p < P; p += 256) {
+        const uint4 u = src[(int64_t)p * (kC / 8)];
+        const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 u = src[q];
-            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 f = __bfloat1622float2(h2[e]);
-                s[q * 8 + 2 * e] += f.x;
-                s[q * 8 + 2 * e + 1] += f.y;
-            }
+        for (int e = 0; e < 4; ++e) {
+            const float2 f = __bfloat1622float2(h2[e]);
+            s[2 * e] += f.x;
+            s[2 * e + 1] += f.y;
         }
     }
 #pragma unroll
-    for (int c = 0; c < kC; ++c) sh[threadIdx.x][c] = s[c];
+    for (int c = 0; c < 8; ++c) sh[row][c0 + c] = s[c];
     __syncthreads();
     for (int off = 128; off > 0; off >>= 1) {
-        if ((int)threadIdx.x < off)
-            for (int c = 0; c < kC; ++c) sh[threadIdx.x][c] += sh[threadIdx.x + off][c];
+        if (row < off)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sh[row][c0 + c] += sh[row + off][c0 + c];
         __syncthreads();
     }
     if (threadIdx.x < kC) pooled[b * kC + threadIdx.x] = sh[0][threadIdx.x] / (float)P;
-    __syncthreads();
     if (threadIdx.x == 0) {
         float v = head[kC];
         for (int c = 0; c < kC; ++c) v += head[c] * (sh[0][c] / (float)P);
@@ -493,11 +540,13 @@ __global__ void head_backward_kernel(int B, int P, const float* pooled, const fl
     __syncthreads();
     if (tid < kC) {
         float gv = 0.f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) gv += dp[b] * pooled[b * kC + tid];
         grad_head[tid] = gv;
     }
     if (tid == kC) {
         float gb = 0.f, l = 0.f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) {
             gb += dp[b];
             const float e = pred[b] - y[b];
@@ -727,7 +776,7 @@ int forward(cnn_model* m, const bf16* x, int batch, cudaStream_t s)
     count_launches(1);
     for (int l = 1; l < kLayers; ++l)
         if (int rc = conv32(m, m->act[l - 1], m->w[l], nullptr, m->act[l], batch, false, s)) return rc;
-    head_forward_kernel<<<batch, 256, 0, s>>>(m->act[kLayers - 1], m->H * m->W, m->master + m->off[kLayers],
+    head_forward_kernel<<<batch, kHeadThreads, 0, s>>>(m->act[kLayers - 1], m->H * m->W, m->master + m->off[kLayers],
                                              m->pooled, m->pred);
     LBM_CUDA(cudaGetLastError());
     count_launches(1);
@@ -756,7 +805,7 @@ int wgrad(cnn_model* m, int l, const bf16* x, const bf16* dy, int batch, cudaStr
         count_launches(1);
     }
     const int n = kC * kp;
-    reduce_partials_kernel<<<(n + 255) / 256, 256, 0, s>>>(m->wpart, nblk, n, m->grad + m->off[l]);
+    reduce_partials_kernel<<<(n + 31) / 32, 256, 0, s>>>(m->wpart, nblk, n, m->grad + m->off[l]);
     LBM_CUDA(cudaGetLastError());
     count_launches(1);
     return LBM_OK;
