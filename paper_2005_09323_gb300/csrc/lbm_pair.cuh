@@ -11,7 +11,8 @@
 // over random states, with and without force, and over every FP32 argument of
 // the reciprocal from 5e-8 to 1e30).
 #pragma once
-#include "lbm_step.cuh"
+#include "lbm_device.cuh"
+#include "step_params.h"
 
 namespace lbm {
 
@@ -146,17 +147,41 @@ __device__ __forceinline__ void cm_collide2(float2 (&g)[9][N], int i, const BgkC
     g[8][i] = fma2(splat(-0.25f), add2(sub2(R12, p5), R22), g[8][i]);
 }
 
-// the periodic channel's collision of every pair
+// the periodic channel's collision of the pair of sites i
+template <int COLL, int N>
+__device__ __forceinline__ void collide_pair(float2 (&g)[9][N], int i, const StepParams& p)
+{
+    if constexpr (COLL == 0)
+        bgk_collide2<N, true>(g, i, p.bgk, splat(p.bgk.om));
+    else
+        cm_collide2<N, true>(g, i, p.bgk, p.cm, splat(p.cm.ws), splat(p.cm.a), splat(p.cm.b));
+}
+
 template <int COLL, int N>
 __device__ __forceinline__ void collide2(float2 (&g)[9][N], const StepParams& p)
 {
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-        if constexpr (COLL == 0)
-            bgk_collide2<N, true>(g, i, p.bgk, splat(p.bgk.om));
-        else
-            cm_collide2<N, true>(g, i, p.bgk, p.cm, splat(p.cm.ws), splat(p.cm.a), splat(p.cm.b));
-    }
+    for (int i = 0; i < N; ++i) collide_pair<COLL>(g, i, p);
+}
+
+// f(pairs, i) on every pair of the V sites of g
+template <int V, typename F>
+__device__ __forceinline__ void on_pairs(float (&g)[9][V], F&& f)
+{
+    float2 h[9][V / 2];
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i) h[q][i] = make_float2(g[q][2 * i], g[q][2 * i + 1]);
+#pragma unroll
+    for (int i = 0; i < V / 2; ++i) f(h, i);
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i) {
+            g[q][2 * i] = h[q][i].x;
+            g[q][2 * i + 1] = h[q][i].y;
+        }
 }
 
 // the open channel's collision of the pair of sites i at the rates om

@@ -31,6 +31,7 @@
 #include <type_traits>
 #include "internal.h"
 #include "lbm_device.cuh"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 
@@ -526,12 +527,20 @@ __device__ __forceinline__ void step_warp(const StepParams& p, const typename Co
     if constexpr (OPEN) {
         // one collision body per site: the rate of a sponge column, else 1/tau
         const bool sponge = x0 + V > p.sx0;
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
+        auto rate = [&](int j) {
             const int x = x0 + j;
-            const float om = sponge && x >= p.sx0 && x < p.nx ? __ldg(p.om_col + x) : p.bgk.om;
-            collide_at<COLL, V>(g, j, p, om);
+            return sponge && x >= p.sx0 && x < p.nx ? __ldg(p.om_col + x) : p.bgk.om;
+        };
+        if constexpr (V % 2 == 0) {
+            on_pairs(g, [&](auto& h, int i) {
+                collide_at2<COLL>(h, i, p, make_float2(rate(2 * i), rate(2 * i + 1)));
+            });
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; ++j) collide_at<COLL, V>(g, j, p, rate(j));
         }
+    } else if constexpr (V % 2 == 0 && S != kFP32) {
+        on_pairs(g, [&](auto& h, int i) { collide_pair<COLL>(h, i, p); });
     } else {
 #pragma unroll
         for (int j = 0; j < V; ++j) collide<COLL, V>(g, j, p);

@@ -90,8 +90,12 @@ __device__ __forceinline__ float rows_sites(const StepParams& p, const typename 
             }
         }
     }
+    if constexpr (V % 2 == 0 && S != kFP32) {
+        on_pairs(g, [&](auto& h, int i) { collide_pair<COLL>(h, i, p); });
+    } else {
 #pragma unroll
-    for (int j = 0; j < V; ++j) collide<COLL, V>(g, j, p);
+        for (int j = 0; j < V; ++j) collide<COLL, V>(g, j, p);
+    }
     float acc = 0.f;
     if (GENERAL && ring) {
         const bool row_solid = y >= p.oy0 && y < p.oy1;

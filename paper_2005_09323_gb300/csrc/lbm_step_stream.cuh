@@ -35,7 +35,7 @@
 // 256), 159 / 203 (16 x 2048 x 512); FP16 central moments 132 / 138.
 #pragma once
 #include "async_copy.cuh"
-#include "lbm_pair.cuh"
+#include "lbm_step.cuh"
 
 namespace lbm {
 
