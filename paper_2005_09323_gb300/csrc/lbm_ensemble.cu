@@ -766,7 +766,7 @@ int stream_variant(int storage)
 }
 
 // the variant of a step call over n_list clones.  A call of four steps and more
-// on a periodic channel streams rows, two steps per pass over memory, if every
+// streams rows, two steps per pass over memory, if every
 // block then has enough rows: a block recomputes two rows of its span, and each
 // of its rows waits on the one before.  Measured on channels of 128 to 2048
 // columns (single steps / streamed, us per step): FP32 BGK 16.6 / 17.1 at 5
@@ -783,11 +783,18 @@ int variant_for(const lbm_ensemble* e, int n_list, int n_steps)
     const int s = stream_variant(c.storage);
     if (e->variant_tuned && vi != s) return vi;
     vi = e->variant_tuned ? default_variant(c.storage) : vi;
-    if (c.open_x || e->observe || n_steps < 4 || s < 0) return vi;
+    if (e->observe || n_steps < 4 || s < 0) return vi;
     if (!vars[s].supports(make_params(e, e->all_dev, n_list, vars[s].vec, 0, 3))) return vi;
-    const int threads = (c.nx + 127) / 128 * 32;
+    const int threads = ((c.open_x ? c.nx - 1 : c.nx) + 127) / 128 * 32;
     const int64_t blocks = (int64_t)(512 / threads) * 152;
-    const int64_t min_rows = c.collision == 0 ? 8 : 12;
+    // (open channels, 513 x 129, the work on their columns included: FP32 central
+    // moments 32.0 / 36.8 us at 7 rows a block, 61.4 / 57.8 at 14; FP32 BGK 57.3 /
+    // 61.4 at 14, 113 / 109 at 27; FP16 central moments 18.9 / 21.3 at 3, 38.1 /
+    // 28.4 at 7, 74.4 / 52.3 at 14; FP16 BGK 35.4 / 25.5 at 7)
+    const int64_t min_rows = !c.open_x                ? (c.collision == 0 ? 8 : 12)
+                             : c.storage != LBM_FP32 ? 6
+                             : c.collision == 1      ? 12
+                                                     : 24;
     return (int64_t)n_list * c.ny >= min_rows * blocks ? s : vi;
 }
 
@@ -842,13 +849,16 @@ int launch_chunk(lbm_ensemble* e, int vi, const int32_t* list_dev, int n_list, i
         s += k;
     }
     auto params = [&](size_t i) {
-        StepParams p = make_params(e, list_dev, n_list, v.vec, first[i], v.kind, chunk);
+        // (the single steps before streamed ones end with the outlet column in place)
+        StepParams p = make_params(e, list_dev, n_list, v.vec, first[i], v.kind,
+                                   v.kind == 3 && first[i] < singles ? singles : chunk);
         p.tb_steps = count[i];
         p.flip = (int32_t)(i & 1);
         return p;
     };
     // an open channel adds the outlet kernel once per chunk, observables their own kernel per step
-    const int launches = (int)first.size() + (e->observe ? chunk : 0) + (e->cfg.open_x ? 1 : 0);
+    const int launches = (int)first.size() + (e->observe ? chunk : 0) +
+                         (e->cfg.open_x && (v.kind != 3 || singles > 0) ? 1 : 0);
     if (!e->use_graphs) {
         for (size_t i = 0; i < first.size(); ++i) {
             cudaError_t err = launch(params(i), e->stream);
@@ -1192,7 +1202,7 @@ int lbm_ensemble_create(const lbm_config* cfg, int32_t n_clones, uint64_t seed, 
     }
     if (e->n_ckpt > 0) { ALLOC(e->ckpt, (size_t)e->clone_stride * e->elem_bytes * n_clones * e->n_ckpt); }
     if (c.open_x) {
-        ALLOC(e->om_col, sizeof(float) * c.nx);
+        ALLOC(e->om_col, sizeof(float) * e->pitch);  // padded: read four columns at a time
         ALLOC(e->inlet_g, sizeof(float) * 9 * c.ny);
         ALLOC(e->open_u, sizeof(float) * 2 * 4 * c.ny * (size_t)n_clones);
     }
@@ -1211,7 +1221,7 @@ int lbm_ensemble_create(const lbm_config* cfg, int32_t n_clones, uint64_t seed, 
     if ((rc = chk(cudaMemsetAsync(e->drag, 0, sizeof(double) * (size_t)n_clones * c.max_steps, e->stream), "memset drag"))) return rc;
     if (c.open_x) {
         // per-column relaxation rate and the inlet populations (FP64, then FP32)
-        std::vector<float> om(c.nx), inlet(9 * (size_t)c.ny);
+        std::vector<float> om(e->pitch, (float)(1.0 / c.tau)), inlet(9 * (size_t)c.ny);
         for (int x = 0; x < c.nx; ++x) om[x] = (float)(1.0 / open_tau(c, x));
         for (int y = 0; y < c.ny; ++y) {
             const double h = c.ny, yy = y + 0.5, u = c.u_in * 4.0 * yy * (h - yy) / (h * h);
@@ -1220,7 +1230,7 @@ int lbm_ensemble_create(const lbm_config* cfg, int32_t n_clones, uint64_t seed, 
                 inlet[(size_t)q * c.ny + y] = (float)(wd(q) * (3.0 * cu + 4.5 * cu * cu - 1.5 * u * u));
             }
         }
-        if ((rc = chk(cudaMemcpyAsync(e->om_col, om.data(), sizeof(float) * c.nx, cudaMemcpyHostToDevice, e->stream), "copy sponge rates"))) return rc;
+        if ((rc = chk(cudaMemcpyAsync(e->om_col, om.data(), sizeof(float) * om.size(), cudaMemcpyHostToDevice, e->stream), "copy sponge rates"))) return rc;
         if ((rc = chk(cudaMemcpyAsync(e->inlet_g, inlet.data(), sizeof(float) * inlet.size(), cudaMemcpyHostToDevice, e->stream), "copy inlet"))) return rc;
         // the copies read pageable host memory: wait before the vectors go
         if ((rc = chk(cudaStreamSynchronize(e->stream), "open-channel tables"))) return rc;

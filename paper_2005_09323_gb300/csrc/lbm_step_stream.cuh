@@ -122,11 +122,16 @@ __device__ __forceinline__ void stream_store(Vec<typename Codec<S>::T, kStreamV>
 // without); the central-moment collision one site at a time, since on pairs its
 // constants and temporaries take registers the row loop does not have (96 bytes
 // of spills, 126 against 127 GLUPS at 64 x 1024 x 256, 123 against 134 at 256 x 512 x 128)
-template <int COLL>
-__device__ __forceinline__ void stream_collide(float2 (&g)[9][kStreamV / 2], const StepParams& p)
+// An open channel's sites relax at their columns' rates om.
+template <int COLL, bool OPEN>
+__device__ __forceinline__ void stream_collide(float2 (&g)[9][kStreamV / 2], const StepParams& p,
+                                               const float2 (&om)[kStreamV / 2])
 {
-    if constexpr (COLL == 0) {
+    if constexpr (COLL == 0 && !OPEN) {
         collide2<0, kStreamV / 2>(g, p);
+    } else if constexpr (OPEN) {
+#pragma unroll
+        for (int i = 0; i < kStreamV / 2; ++i) collide_at2<COLL>(g, i, p, om[i]);
     } else {
         float f[9][kStreamV];
 #pragma unroll
@@ -156,6 +161,15 @@ __device__ __forceinline__ void stream_collide(float2 (&g)[9][kStreamV / 2], con
 // partials these are: 4 for FP32, 8 for 16-bit storage.
 template <int S>
 constexpr int kStreamGroup = S == kFP32 ? 4 : 8;
+
+// the rates of the columns x .. x + 3 of an open channel
+__device__ __forceinline__ void stream_rates(const StepParams& p, int x, float2 (&om)[kStreamV / 2])
+{
+#pragma unroll
+    for (int i = 0; i < kStreamV / 2; ++i)
+        om[i] = make_float2(x + 2 * i < p.nx ? __ldg(p.om_col + x + 2 * i) : p.bgk.om,
+                            x + 2 * i + 1 < p.nx ? __ldg(p.om_col + x + 2 * i + 1) : p.bgk.om);
+}
 
 template <int S>
 struct StreamRegion {
@@ -212,7 +226,9 @@ struct StreamRegion {
 // columns xl and xr.  Streaming with bounce-back, collision, rest state of solid
 // sites; returns the group's momentum exchange with the obstacle so far: where
 // two threads share a group, the odd lane continues the sum of the lane before.
-template <int S, bool SCALED, int COLL>
+// OPEN: also the bars of an open channel's grid and its inlet column (sites past
+// the last column are left at rest; the outlet column is the caller's).
+template <int S, bool SCALED, int COLL, bool OPEN, bool DRAG = true>
 __device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (&g)[9][kStreamV / 2], int x, int y,
                                                    const typename Codec<S>::T* base, int qs, int rs, int yc, int xc,
                                                    int xl, int xr)
@@ -220,11 +236,21 @@ __device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (
     using T = typename Codec<S>::T;
     using K = Carry<S, SCALED>;
     constexpr int V = kStreamV;
-    uint32_t cols = 0;  // bit i: site x - 1 + i is in the obstacle's columns
+    uint32_t cols = 0, bars = 0;  // bit i: site x - 1 + i is in the obstacle's, the grid's columns
 #pragma unroll
-    for (int i = 0; i < V + 2; ++i) cols |= (x - 1 + i >= p.ox0 && x - 1 + i < p.ox1 ? 1u : 0u) << i;
-    // the sites beyond a periodic seam: columns 0 and nx - 1 are never solid
-    auto solid_row = [&](int r) { return r >= p.oy0 && r < p.oy1; };
+    for (int i = 0; i < V + 2; ++i) {
+        cols |= (x - 1 + i >= p.ox0 && x - 1 + i < p.ox1 ? 1u : 0u) << i;
+        if (OPEN) bars |= (x - 1 + i >= p.gx0 && x - 1 + i < p.gx1 ? 1u : 0u) << i;
+    }
+    // (the sites beyond a periodic seam: columns 0 and nx - 1 are never solid)
+    auto square_row = [&](int r) { return r >= p.oy0 && r < p.oy1 ? cols : 0u; };
+    uint32_t solid[3];  // solid sites among x - 1 .. x + 4 of rows y - 1, y, y + 1
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int r = y - 1 + d;
+        solid[d] = square_row(r);
+        if (OPEN && bars != 0u && r >= 0 && r < p.ny && r % p.gperiod >= p.ggap) solid[d] |= bars;
+    }
     Vec<T, V> v[9];
     T e[9];
 #pragma unroll
@@ -252,32 +278,39 @@ __device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (
             else
                 f[q][j] = d[j];
         }
-        if (q > 0 && solid_row(y - cy(q)) && (cols >> (1 - cx(q)) & ((1u << V) - 1u))) {
+        const uint32_t back = q > 0 ? solid[1 - cy(q)] >> (1 - cx(q)) & ((1u << V) - 1u) : 0u;
+        if (back != 0u) {
             const Vec<T, V> o = *reinterpret_cast<const Vec<T, V>*>(base + opp(q) * qs + yc * rs + xc);
 #pragma unroll
             for (int j = 0; j < V; ++j)
-                if (cols >> (j + 1 - cx(q)) & 1u) f[q][j] = K::in(o.e[j], wf(q), p.inv_scale);
+                if (back >> j & 1u) f[q][j] = K::in(o.e[j], wf(q), p.inv_scale);
         }
 #pragma unroll
         for (int i = 0; i < V / 2; ++i) g[q][i] = make_float2(f[q][2 * i], f[q][2 * i + 1]);
     }
-    collide2<COLL, V / 2>(g, p);
+    if constexpr (OPEN) {
+        float2 om[V / 2];
+        stream_rates(p, x, om);
+        stream_collide<COLL, true>(g, p, om);
+    } else {
+        collide2<COLL, V / 2>(g, p);
+    }
     auto sum = [&](float acc) {
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-            const bool solid = solid_row(y) && (cols >> (j + 1) & 1u);
+            const bool inside = square_row(y) >> (j + 1) & 1u;
 #pragma unroll
             for (int q = 1; q < 9; ++q) {
                 if (cx(q) == 0) continue;
                 const float gq = j & 1 ? g[q][j / 2].y : g[q][j / 2].x;
-                if (!solid && solid_row(y + cy(q)) && (cols >> (j + 1 + cx(q)) & 1u))
+                if (!inside && (square_row(y + cy(q)) >> (j + 1 + cx(q)) & 1u))
                     acc += 2.0f * (float)cx(q) * (wf(q) + gq);
             }
         }
         return acc;
     };
-    float acc = sum(0.f);
-    if constexpr (kStreamGroup<S> > V) {
+    float acc = DRAG ? sum(0.f) : 0.f;
+    if constexpr (DRAG && kStreamGroup<S> > V) {
         const float before = __shfl_up_sync(0xffffffffu, acc, 1);
         if (threadIdx.x & 1) acc = sum(before);
     }
@@ -285,7 +318,11 @@ __device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (
     for (int q = 0; q < 9; ++q)
 #pragma unroll
         for (int j = 0; j < V; ++j)
-            if (solid_row(y) && (cols >> (j + 1) & 1u)) (j & 1 ? g[q][j / 2].y : g[q][j / 2].x) = 0.f;  // rest: f = w
+            if (solid[1] >> (j + 1) & 1u || (OPEN && x + j >= p.nx))
+                (j & 1 ? g[q][j / 2].y : g[q][j / 2].x) = 0.f;  // rest: f = w
+    if (OPEN && x == 0)
+#pragma unroll
+        for (int q = 0; q < 9; ++q) g[q][0].x = __ldg(p.inlet_g + q * p.ny + y);
     return acc;
 }
 
@@ -322,9 +359,9 @@ struct StreamGroups {
     }
 };
 
-// both steps of the obstacle's region for every listed clone, in chunks of rows
-// over the blocks, and the drag partials of its rows
-template <int S, bool SCALED, int COLL>
+// both steps of the obstacle's region for every listed clone, in chunks of R
+// rows over the blocks, and the drag partials of its rows
+template <int S, bool SCALED, int COLL, bool OPEN>
 __device__ __noinline__ void stream_obstacle(const StepParams& p, unsigned char* smem, int R)
 {
     using T = typename Codec<S>::T;
@@ -352,8 +389,9 @@ __device__ __noinline__ void stream_obstacle(const StepParams& p, unsigned char*
             const bool in = i < first.total * H;
             const int h = i % H * V, x = rg.wrap(rg.l0 + gi) * G + h;
             float2 g[9][V / 2];
-            const float acc = stream_site_group<S, SCALED, COLL>(p, g, x, y, src, plane, p.pitch, y, x,
-                                                                 x == 0 ? nx - 1 : x - 1, x + V == nx ? 0 : x + V);
+            const float acc = stream_site_group<S, SCALED, COLL, OPEN>(
+                p, g, x, y, src, plane, p.pitch, y, x, x == 0 ? nx - 1 : x - 1,
+                OPEN ? min(x + V, nx - 1) : (x + V == nx ? 0 : x + V));
             if (in) {
 #pragma unroll
                 for (int q = 0; q < 9; ++q) {
@@ -373,8 +411,8 @@ __device__ __noinline__ void stream_obstacle(const StepParams& p, unsigned char*
             const int gi = rg.wrap(gg - rg.l0), h = i % H * V, x = rg.wrap(gg) * G + h, lx = gi * G + h;
             float2 g[9][V / 2];
             // (beyond the tile's columns only where it is the whole row)
-            const float acc = stream_site_group<S, SCALED, COLL>(p, g, x, y, tile, tq, tw, y - la, lx,
-                                                                 lx == 0 ? tw - 1 : lx - 1, lx + V == tw ? 0 : lx + V);
+            const float acc = stream_site_group<S, SCALED, COLL, OPEN>(
+                p, g, x, y, tile, tq, tw, y - la, lx, lx == 0 ? tw - 1 : lx - 1, lx + V == tw ? 0 : lx + V);
             if (in) {
 #pragma unroll
                 for (int q = 0; q < 9; ++q) {
@@ -414,6 +452,190 @@ __device__ __noinline__ void stream_obstacle(const StepParams& p, unsigned char*
     }
 }
 
+// Open channels (Sec. 2).  The stream itself takes 40 us per step and 64 x 513 x
+// 129 nodes in FP32 (31 in FP16), the columns below, 8 % of the sites, another 17
+// (21): about 1700 instructions for four sites and a step with all their cases.
+// Bars and inlet inside the stream instead, in the warp that holds them, made
+// every row wait for that warp (67 and 54 us in all, against 58 and 52).
+//
+// Columns of an open channel whose two steps the row stream does not know, in
+// groups as above, over all rows: around the inlet column (range 0), the grid of
+// bars (1), and columns nx - 3 .. nx - 1 before and at the outlet (2; it pulls
+// from an outlet column that the velocities of three rows give).
+template <int S>
+struct StreamColumns {
+    static constexpr int G = kStreamGroup<S>;
+    int g0[3], g1[3], total;  // [g0, g1); groups of a row
+    __host__ __device__ explicit StreamColumns(const StepParams& p)
+    {
+        total = (p.nx - 1) / G + 1;
+        g0[0] = 0;
+        g1[0] = 1;
+        g0[1] = g1[1] = 0;
+        if (p.gx1 > p.gx0) {
+            g0[1] = p.gx0 >= 2 ? (p.gx0 - 2) / G : 0;
+            g1[1] = (p.gx1 + 1) / G + 1;
+            if (g0[1] == 0) g1[0] = 0;  // the grid's range holds the inlet's
+        }
+        g0[2] = (p.nx - 3) / G;
+        g1[2] = total;
+    }
+    __host__ __device__ bool has(int g) const
+    {
+        return (g >= g0[0] && g < g1[0]) || (g >= g0[1] && g < g1[1]) || g >= g0[2];
+    }
+    __host__ __device__ static int halo(int r) { return r == 2 ? 3 : 1; }
+    // groups of the intermediate step: one more on either side
+    __host__ __device__ int l0(int r) const { return g0[r] > 0 ? g0[r] - 1 : 0; }
+    __host__ __device__ int l1(int r) const { return g1[r] < total ? g1[r] + 1 : total; }
+    __host__ __device__ size_t bytes(int r, int rows) const
+    {
+        return (size_t)9 * (rows + 2 * halo(r)) * (l1(r) - l0(r)) * G * sizeof(typename Codec<S>::T) +
+               (r == 2 ? 4 * sizeof(float) * (rows + 2) : 0);
+    }
+    // rows of a chunk: two passes of the block over the intermediate step's
+    // groups, or what the shared memory holds; 0: not even one row
+    __host__ __device__ int chunk(int r, int threads, size_t smem, int ny) const
+    {
+        int n = 2 * threads / ((l1(r) - l0(r)) * (G / kStreamV)) - 2 * halo(r);
+        n = n < 1 ? 1 : (n > ny ? ny : n);
+        while (n > 0 && bytes(r, n) > smem) --n;
+        return n;
+    }
+    // the obstacle's region must keep to its own groups, and the ranges be apart
+    __host__ __device__ bool apart(const StreamRegion<S>& rg) const
+    {
+        if (g1[1] > g0[2] || g1[0] > g0[2]) return false;
+        if (rg.ng == 0) return true;
+        const int a = rg.g0, b = rg.g0 + rg.ng;
+        return a >= 1 && a >= g1[0] && b <= g0[2] && (g1[1] == g0[1] || b <= g0[1] || a >= g1[1]) &&
+               rg.nl < rg.groups;
+    }
+};
+
+// both steps of rows [ra, rb) of column range r for listed clone li
+template <int S, bool SCALED, int COLL>
+__device__ __noinline__ void stream_columns(const StepParams& p, unsigned char* smem, int li, int r, int ra, int rb)
+{
+    using T = typename Codec<S>::T;
+    using K = Carry<S, SCALED>;
+    constexpr int V = kStreamV, G = kStreamGroup<S>, H = G / V;
+    const StreamColumns<S> cols(p);
+    const int nx = p.nx, ny = p.ny, plane = (int)p.plane, tid = threadIdx.x;
+    const bool outlet = r == 2;
+    const int c = p.clone_list[li], cur = p.parity[c] ^ p.flip;
+    const T* src = static_cast<const T*>(cur ? p.buf1 : p.buf0) + (int64_t)c * p.clone_stride;
+    T* dst = static_cast<T*>(cur ? p.buf0 : p.buf1) + (int64_t)c * p.clone_stride;
+    const int hh = cols.halo(r), la = max(ra - hh, 0), lb = min(rb + hh, ny);
+    const int xa = cols.l0(r) * G, tw = (cols.l1(r) - cols.l0(r)) * G, tq = (lb - la) * tw;
+    T* const tile = reinterpret_cast<T*>(smem);                                   // [q][row][tw], column xa first
+    float* const uv = reinterpret_cast<float*>(smem + (size_t)9 * tq * sizeof(T));  // [4][rows + 2]: as p.open_u
+    const int n1 = (lb - la) * (tw / V);
+    for (int i = tid; (i & ~31) < n1; i += blockDim.x) {
+        const int k = min(i, n1 - 1), y = la + k / (tw / V), x = xa + k % (tw / V) * V;
+        float2 g[9][V / 2];
+        stream_site_group<S, SCALED, COLL, true, false>(p, g, x, y, src, plane, p.pitch, y, x, max(x - 1, 0),
+                                                 min(x + V, nx - 1));
+        if (i < n1)
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                Vec<T, V> o;
+                stream_store<S, SCALED>(o, g[q], wf(q), p.scale);
+                *reinterpret_cast<Vec<T, V>*>(tile + q * tq + (y - la) * tw + x - xa) = o;
+            }
+    }
+    __syncthreads();
+    // velocity of a stored node of the tile, as the step kernel leaves it in p.open_u
+    auto velocity = [&](int x, int y, float& u, float& v) {
+        float h[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) h[q] = K::in(tile[q * tq + (y - la) * tw + x - xa], wf(q), p.inv_scale);
+        open_velocity9(h, u, v);
+    };
+    if (outlet) {  // the outlet column of the intermediate step
+        const int oa = max(ra - 2, 0), ob = min(rb + 2, ny);
+        for (int y = oa + tid; y < ob; y += blockDim.x) {
+            const int ym = max(y - 1, 0), yp = min(y + 1, ny - 1);
+            OutletU a;
+            velocity(nx - 2, y, a.u2, a.v2);
+            velocity(nx - 3, y, a.u3, a.v3);
+            velocity(nx - 2, ym, a.u2m, a.v2m);
+            velocity(nx - 3, ym, a.u3m, a.v3m);
+            velocity(nx - 2, yp, a.u2p, a.v2p);
+            velocity(nx - 3, yp, a.u3p, a.v3p);
+            a.two = yp - ym == 2;
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                tile[q * tq + (y - la) * tw + nx - 1 - xa] =
+                    K::out(outlet_g(a, (float)cx(q), (float)cy(q), wf(q), p.bc_pre), wf(q), p.scale);
+        }
+        __syncthreads();
+    }
+    // ---- second step; for the outlet also of the rows next to the chunk
+    const int pa = outlet ? max(ra - 1, 0) : ra, pb = outlet ? min(rb + 1, ny) : rb, un = pb - pa;
+    const int gw = (cols.g1[r] - cols.g0[r]) * H, n2 = un * gw;
+    // the register-staged kernel's last vector leaves the row's padding at rest
+    const bool pads = (nx - 1) % (32 * G) != 0;
+    for (int i = tid; (i & ~31) < n2; i += blockDim.x) {
+        const int k = min(i, n2 - 1), y = pa + k / gw, x = cols.g0[r] * G + k % gw * V, lx = x - xa;
+        float2 g[9][V / 2];
+        stream_site_group<S, SCALED, COLL, true, false>(p, g, x, y, tile, tq, tw, y - la, lx, max(lx - 1, 0),
+                                                 min(lx + V, tw - 1));
+        if (i >= n2) continue;
+        if (outlet)
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                if (x + j == nx - 2 || x + j == nx - 3) {
+                    float h[9], u, v;
+#pragma unroll
+                    for (int q = 0; q < 9; ++q)
+                        h[q] = K::in(K::out(j & 1 ? g[q][j / 2].y : g[q][j / 2].x, wf(q), p.scale), wf(q), p.inv_scale);
+                    open_velocity9(h, u, v);
+                    float* o = uv + (x + j == nx - 2 ? 0 : 2) * un + y - pa;
+                    o[0] = u;
+                    o[un] = v;
+                }
+        if (y < ra || y >= rb) continue;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            Vec<T, V> o;
+            stream_store<S, SCALED>(o, g[q], wf(q), p.scale);
+            T* to = dst + q * plane + y * p.pitch + x;
+            if (x + V < nx) {
+                st_stream<T, V>(to, o);
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (x + j < nx - 1 || (x + j >= nx && pads)) to[j] = o.e[j];
+            }
+        }
+    }
+    __syncthreads();
+    if (outlet)
+        for (int y = ra + tid; y < rb; y += blockDim.x) {
+            const int k = y - pa, km = max(y - 1, 0) - pa, kp = min(y + 1, ny - 1) - pa;
+            OutletU a;
+            a.u2 = uv[k];
+            a.v2 = uv[un + k];
+            a.u3 = uv[2 * un + k];
+            a.v3 = uv[3 * un + k];
+            a.u2m = uv[km];
+            a.v2m = uv[un + km];
+            a.u3m = uv[2 * un + km];
+            a.v3m = uv[3 * un + km];
+            a.u2p = uv[kp];
+            a.v2p = uv[un + kp];
+            a.u3p = uv[2 * un + kp];
+            a.v3p = uv[3 * un + kp];
+            a.two = kp - km == 2;
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                dst[q * plane + y * p.pitch + nx - 1] =
+                    K::out(outlet_g(a, (float)cx(q), (float)cy(q), wf(q), p.bc_pre), wf(q), p.scale);
+        }
+    __syncthreads();
+}
+
 // keeps the compiler from holding the nine plane offsets of the loads and of
 // the stores in registers across the row loop (they cost one instruction each)
 __device__ __forceinline__ int stream_opaque(int v)
@@ -446,7 +668,7 @@ struct StreamWarpSmem {
     VT up[2][3][32];  // directions 2, 5, 6 of the intermediate step, by row mod 2
 };
 
-template <int S, bool SCALED, int COLL>
+template <int S, bool SCALED, int COLL, bool OPEN>
 __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const __grid_constant__ StepParams p)
 {
     using T = typename Codec<S>::T;
@@ -467,22 +689,54 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
     // about as long as two of its rows
     const int rows = p.n_list * ny, grid = gridDim.x, bytes = nwarp * (int)sizeof(StreamWarpSmem<S>);
     const int chunk = rg.ng > 0 ? rg.chunk(blockDim.x, bytes, grid / (kStreamMaxThreads / blockDim.x), p.n_list) : 1;
-    const int items = p.n_list * ((rg.r1 - rg.r0 + chunk - 1) / chunk), cost = rows >= 4 * grid ? 2 : 0;
+    const int squares = p.n_list * ((rg.r1 - rg.r0 + chunk - 1) / chunk);
+    int items = squares, range_rows[3] = {1, 1, 1}, range_chunks[3] = {0, 0, 0};
+    if constexpr (OPEN) {
+        const StreamColumns<S> cols(p);
+        for (int r = 0; r < 3; ++r)
+            if (cols.g1[r] > cols.g0[r]) {
+                range_rows[r] = cols.chunk(r, blockDim.x, bytes, ny);
+                range_chunks[r] = (ny + range_rows[r] - 1) / range_rows[r];
+                items += p.n_list * range_chunks[r];
+            }
+    }
+    const int cost = rows >= 8 * grid ? 2 : 0;
     auto span = [&](int b) {
         return (int)((rows + (int64_t)cost * items) * b / grid) - cost * (items / grid * b + min(b, items % grid));
     };
     const int s0 = span(blockIdx.x), s1 = span(blockIdx.x + 1);
     const int x0 = tid * V;
-    const bool active = x0 < nx;
-    const int xr = active ? x0 : nx - V;
-    const bool first = lane == 0, last = lane == 31 || x0 + V >= nx;  // sites at the edges of the warp's columns
+    // an open channel's columns from nx - 1 on are not streamed (its rows' padding
+    // is read and feeds only sites computed apart)
+    const bool active = OPEN ? x0 < nx - 1 : x0 < nx;
+    const int xr = OPEN || active ? x0 : nx - V;
+    const bool first = lane == 0, last = lane == 31 || (!OPEN && x0 + V >= nx);  // at the edges of the warp's columns
     const int wl = warp == 0 ? nwarp - 1 : warp - 1, wr = warp + 1 == nwarp ? 0 : warp + 1;
     const bool apart = rg.ng > 0 && rg.has(x0 / kStreamGroup<S>);  // in the obstacle's columns: computed by stream_obstacle
+    const bool streamed = active && !(OPEN && StreamColumns<S>(p).has(x0 / kStreamGroup<S>));
+    auto collide_row = [&](float2 (&g)[9][V / 2]) {
+        float2 om[V / 2] = {};
+        if constexpr (OPEN) {
+            const float4 o = __ldg(reinterpret_cast<const float4*>(p.om_col + x0));  // padded to the row pitch
+            om[0] = make_float2(o.x, o.y);
+            om[1] = make_float2(o.z, o.w);
+        }
+        stream_collide<COLL, OPEN>(g, p, om);
+    };
 
     if (tid < 4 * nwarp) mbar_init(smem_addr(&edge_ready[tid & 3][tid >> 2]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     __syncthreads();
-    if (rg.ng > 0) stream_obstacle<S, SCALED, COLL>(p, smem, chunk);
+    if (rg.ng > 0) stream_obstacle<S, SCALED, COLL, OPEN>(p, smem, chunk);
+    if constexpr (OPEN) {
+        for (int i = blockIdx.x; i < items; i += grid) {  // after the obstacle's chunks, the column ranges'
+            int k = i - squares, r = 0;
+            if (k < 0) continue;
+            while (k >= p.n_list * range_chunks[r]) k -= p.n_list * range_chunks[r++];
+            const int ra = k % range_chunks[r] * range_rows[r];
+            stream_columns<S, SCALED, COLL>(p, smem, k / range_chunks[r], r, ra, min(ra + range_rows[r], ny));
+        }
+    }
 
     StreamWalk w{s0, s1, ny};
     if (!w.piece()) return;
@@ -497,7 +751,11 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
     // fetches, and that value's column (16-bit: the 4 bytes that hold it)
     const int eq = lane == 0 ? 1 : lane == 1 ? 5 : lane == 2 ? 8 : lane == 3 ? 3 : lane == 4 ? 6 : 7;
     const int xw = warp * 32 * V;
-    const int xe = lane < 3 ? (xw == 0 ? nx - 1 : xw - 1) : (xw + 32 * V >= nx ? 0 : xw + 32 * V);
+    auto edge_col = [&](bool left) {
+        if (OPEN) return left ? max(xw - 1, 0) : min(xw + 32 * V, nx - 1);
+        return left ? (xw == 0 ? nx - 1 : xw - 1) : (xw + 32 * V >= nx ? 0 : xw + 32 * V);
+    };
+    const int xe = edge_col(lane < 3);
     auto load_row = [&](int stage) {
         if (more) {
             const T* src = from_clone;
@@ -526,7 +784,7 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
     };
     for (int i = 0; i < kStreamStages; ++i) load_row(i);
     auto beyond = [&](int stage, int i) {
-        const int off = sizeof(T) == 2 ? ((i < 3 ? (xw == 0 ? nx - 1 : xw - 1) : 0) & 1) : 0;
+        const int off = sizeof(T) == 2 ? edge_col(i < 3) & 1 : 0;
         return reinterpret_cast<const T*>(&ws.beyond[stage][i])[off];
     };
 
@@ -578,7 +836,7 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
                 __syncwarp();
                 load_row(stage);  // every lane has read the stage
                 stage = stage + 1 == kStreamStages ? 0 : stage + 1;
-                stream_collide<COLL>(g, p);
+                collide_row(g);
                 auto store = [&](VT& o, int q) { stream_store<S, SCALED>(o, g[q], wf(q), p.scale); };
                 store(C0, 0);
                 store(C1, 1);
@@ -594,7 +852,7 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
                     edge[slot][1][warp] = C6.e[0];
                     edge[slot][2][warp] = C7.e[0];
                 }
-                if (last && active) {
+                if (last && (OPEN || active)) {
                     edge[slot][3][warp] = C1.e[V - 1];
                     edge[slot][4][warp] = C5.e[V - 1];
                     edge[slot][5][warp] = C8.e[V - 1];
@@ -655,8 +913,8 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
                     stream_own<S, SCALED, 7>(g, C7, p.inv_scale);
                     stream_own<S, SCALED, 8>(g, C8, p.inv_scale);
                 }
-                stream_collide<COLL>(g, p);
-                if (active && !(apart && yo >= rg.r0 && yo < rg.r1)) {
+                collide_row(g);
+                if (streamed && !(apart && yo >= rg.r0 && yo < rg.r1)) {
                     const int plane = stream_opaque((int)p.plane);
                     T* out = dst + yo * p.pitch + x0;
 #pragma unroll
@@ -681,45 +939,75 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
     } while (w.piece());
 }
 
-// whole rows of at most 2048 sites in a block; periodic channels
+// threads of a block: a row's columns, in warps (an open channel's without its outlet column)
+inline int stream_threads(const StepParams& p)
+{
+    return ((p.open ? p.nx - 1 : p.nx) + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
+}
+
+// whole rows of at most 2048 sites in a block, the work apart in its shared
+// memory; in an open channel the column ranges and the obstacle's region apart
 template <int S>
 bool stream_supported(const StepParams& p)
 {
-    const int threads = (p.nx + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
+    const int threads = stream_threads(p);
+    const size_t smem = threads / 32 * sizeof(StreamWarpSmem<S>);
     const StreamRegion<S> rg(p);
-    return rg.bytes(2) <= threads / 32 * sizeof(StreamWarpSmem<S>) && !p.open && p.nx % kStreamGroup<S> == 0 && threads <= kStreamMaxThreads &&
-           (int64_t)p.n_list * p.ny < ((int64_t)1 << 31);
+    if (threads > kStreamMaxThreads || rg.bytes(2) > smem || (int64_t)p.n_list * p.ny >= ((int64_t)1 << 31)) return false;
+    if (!p.open) return p.nx % kStreamGroup<S> == 0;
+    const StreamColumns<S> cols(p);
+    if (p.nx < 32 || !cols.apart(rg)) return false;
+    for (int r = 0; r < 3; ++r)
+        if (cols.g1[r] > cols.g0[r] && cols.chunk(r, threads, smem, p.ny) < 1) return false;
+    return true;
 }
 
-template <int S, bool SCALED, int COLL>
+template <int S, bool SCALED, int COLL, bool OPEN>
 cudaError_t launch_stream_kernel(const StepParams& p, cudaStream_t s)
 {
-    const int threads = (p.nx + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
+    const int threads = stream_threads(p);
     const int ctas = kStreamMaxThreads / threads;  // per SM: the 512 threads that 128 registers leave room for
     const size_t smem = threads / 32 * sizeof(StreamWarpSmem<S>);
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t rows = (int64_t)p.n_list * p.ny;
     const int grid = (int)(rows < (int64_t)ctas * sms ? rows : (int64_t)ctas * sms);
-    const cudaError_t e = cudaFuncSetAttribute(step_stream_kernel<S, SCALED, COLL>,
+    const cudaError_t e = cudaFuncSetAttribute(step_stream_kernel<S, SCALED, COLL, OPEN>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)(kStreamMaxThreads / 32 * sizeof(StreamWarpSmem<S>)));
     if (e != cudaSuccess) return e;
-    step_stream_kernel<S, SCALED, COLL><<<grid, threads, smem, s>>>(p);
+    step_stream_kernel<S, SCALED, COLL, OPEN><<<grid, threads, smem, s>>>(p);
     return cudaGetLastError();
 }
 
 // one launch of two steps, or of a single one by the register-staged kernel
 // with the same drag segments
-template <int S>
-cudaError_t launch_stream(const StepParams& p, cudaStream_t s)
+template <int S, bool OPEN>
+cudaError_t launch_stream_of(const StepParams& p, cudaStream_t s)
 {
-    if (p.tb_steps == 1) return launch_step<S, kStreamGroup<S>, 4>(p, s);
+    if (p.tb_steps == 1) {
+        if constexpr (OPEN)
+            return launch_step_open<S, kStreamGroup<S>, 4>(p, s);
+        else
+            return launch_step<S, kStreamGroup<S>, 4>(p, s);
+    }
     if (!stream_supported<S>(p) || p.tb_steps != 2) return cudaErrorInvalidValue;
     const bool scaled = S != kFP32 && p.scale != 1.0f;
     if (p.coll == 1)
-        return scaled ? launch_stream_kernel<S, S != kFP32, 1>(p, s) : launch_stream_kernel<S, false, 1>(p, s);
-    return scaled ? launch_stream_kernel<S, S != kFP32, 0>(p, s) : launch_stream_kernel<S, false, 0>(p, s);
+        return scaled ? launch_stream_kernel<S, S != kFP32, 1, OPEN>(p, s) : launch_stream_kernel<S, false, 1, OPEN>(p, s);
+    return scaled ? launch_stream_kernel<S, S != kFP32, 0, OPEN>(p, s) : launch_stream_kernel<S, false, 0, OPEN>(p, s);
+}
+
+template <int S>
+cudaError_t launch_stream(const StepParams& p, cudaStream_t s)
+{
+    return launch_stream_of<S, false>(p, s);
+}
+
+template <int S>
+cudaError_t launch_stream_open(const StepParams& p, cudaStream_t s)
+{
+    return launch_stream_of<S, true>(p, s);
 }
 
 }  // namespace lbm

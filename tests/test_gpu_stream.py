@@ -69,6 +69,29 @@ def test_stream_is_the_single_step_bit_for_bit(L, storage, shift, collision):
         assert all(np.array_equal(x, y) for x, y in zip(a[1], b[1])), (nx, ny)
 
 
+OPEN_SHAPES = [  # clones, nx, ny, obstacle, grid, sponge columns, step counts
+    (3, 203, 37, (90, 11, 9, 14), (16, 8, 8, 8), 50, (4, 5, 6, 7)),
+    (2, 64, 12, (0, 0, 0, 0), (0, 0, 0, 0), 16, (8,)),
+    (7, 513, 33, (248, 9, 16, 9), (16, 8, 8, 8), 128, (9,)),
+    (4, 517, 129, (248, 56, 16, 16), (2, 8, 8, 8), 128, (13, 4)),  # the grid at the inlet; padded last vector
+    (5, 131, 17, (60, 5, 4, 4), (0, 0, 0, 0), 0, (9, 4)),
+    (2, 1025, 60, (500, 20, 20, 20), (30, 10, 6, 6), 200, (12,)),
+    (3, 512, 40, (200, 0, 30, 9), (5, 3, 4, 4), 100, (8,)),        # the square on a wall
+]
+
+
+@pytest.mark.parametrize("storage,shift", [("fp32", 0), ("fp16", 3), ("bf16", 0)])
+@pytest.mark.parametrize("collision", ["bgk", "cm"])
+def test_open_stream_is_the_single_step_bit_for_bit(L, storage, shift, collision):
+    for n, nx, ny, ob, grid, sponge, steps in OPEN_SHAPES:
+        cfg = L.config(nx, ny, obstacle=ob, tau=0.56, storage=storage, shift_exp=shift, max_steps=64, open_x=1,
+                       u_in=0.05, grid=grid, sponge_len=sponge, sponge_tau=0.9, collision=collision, omega_bulk=1.1,
+                       omega_3=0.9, omega_4=1.2)
+        a, b = (run(L, cfg, n, steps, variant(L, storage, k)) for k in (0, 3))
+        assert np.array_equal(a[0], b[0]), (nx, ny)
+        assert all(np.array_equal(x, y) for x, y in zip(a[1], b[1])), (nx, ny)
+
+
 def test_default_streams_large_calls_only(L):
     """48 clones of 512 x 128 (10 rows a block) stream: 8 steps in 4 launches, as
     the single steps bit for bit; 16 clones step singly; so does a call of three
