@@ -295,8 +295,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         int k = 0;
         for (int ct = blockIdx.x; ct < sh.n_ct; ct += gridDim.x, ++k) {
             const int ab = k & 1;
-            if (!mbar_wait_cycles(smem_addr(&accf[ab]), (k >> 1) & 1, kTcWaitCycles)) abort_flag = 1;
-            if (abort_flag) break;
+            const bool ok = mbar_wait_cycles(smem_addr(&accf[ab]), (k >> 1) & 1, kTcWaitCycles);
+            if (!__all_sync(0xffffffffu, ok && !abort_flag)) {  // the warp goes on, or stops, as one
+                abort_flag = 1;
+                break;
+            }
             tc_fence_after();
             int b, y0, x0;
             tile_origin(sh, ct, b, y0, x0);
@@ -354,7 +357,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 constexpr int kRowSlots = 12;                         // input-row ring
 constexpr int kRowPairSlots = kRowSlots / 2;          // its pairs (one full / empty barrier each)
 constexpr int kRowBufs = 4;                           // accumulators in tensor memory, 128 columns apart
-constexpr int kRowPairBufs = kRowBufs / 2;            // accumulator pairs (one dfull / dfree barrier each)
+constexpr int kRowPairBufs = kRowBufs / 2;            // accumulator pairs (one dfree barrier each)
+// Barriers for accumulator pairs that are ready, pair p on barrier p mod kRowDone.
+// A parity wait for phase f passes at once while phase f - 1 is still open, and an
+// epilogue warpgroup does not wait for the pairs between two of its output rows:
+// from its last pair to its next it skips up to 4 output rows' and 4 runs' input
+// rows, 5 pairs.  With one barrier per accumulator pair (2) a warpgroup whose first
+// output row came after the end of a run of 1 to 3 rows did not wait at all: it read
+// accumulators before their MMAs and freed slots that were not loaded, which faulted
+// (64 x 256 inputs, batch 14; 32 x 128, batch 64).
+constexpr int kRowDone = 8;
 constexpr int kRowEpi = 4;                            // epilogue warpgroups: output rows k = e mod kRowEpi
 constexpr int kRowThreads = 64 + 128 * kRowEpi;
 constexpr uint32_t kRowCols = 512;
@@ -447,7 +459,7 @@ __global__ void __launch_bounds__(kRowThreads, 1)
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[kRowPairSlots];   // per pair of input rows
     __shared__ __align__(8) uint64_t empty[kRowPairSlots];
-    __shared__ __align__(8) uint64_t dfull[kRowPairBufs];   // per pair of accumulators
+    __shared__ __align__(8) uint64_t dfull[kRowDone];       // per pair of accumulators in the ring of kRowDone
     __shared__ __align__(8) uint64_t dfree[kRowPairBufs];
     __shared__ __align__(8) uint64_t done;
     __shared__ uint32_t tmem_slot;
@@ -470,9 +482,9 @@ __global__ void __launch_bounds__(kRowThreads, 1)
             mbar_init(smem_addr(&empty[i]), 2);  // one arrival per input row of the pair
         }
         for (int i = 0; i < kRowPairBufs; ++i) {
-            mbar_init(smem_addr(&dfull[i]), 1);
             mbar_init(smem_addr(&dfree[i]), 24);  // 3 readers x 4 warps per accumulator
         }
+        for (int i = 0; i < kRowDone; ++i) mbar_init(smem_addr(&dfull[i]), 1);
         mbar_init(smem_addr(&done), 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -567,7 +579,7 @@ __global__ void __launch_bounds__(kRowThreads, 1)
                     for (int j = 0; j < 6; ++j) umma_f16_n96(d, ad[j] + so, bd[j], j != 0);
                 }
                 // both D ready for the epilogue, which also frees the input slots
-                umma_commit(smem_addr(&dfull[pb]));
+                umma_commit(smem_addr(&dfull[(sq >> 1) % kRowDone]));
                 if (++ps == kRowPairSlots) {
                     ps = 0;
                     fpar ^= 1u;
@@ -598,15 +610,16 @@ __global__ void __launch_bounds__(kRowThreads, 1)
             ++n;
             if (k++ % kRowEpi != e) return true;
             // the pairs of input rows sq[0..2] (D of pair p in accumulator pair p mod 2)
-            for (int j = 0; j < 3; ++j) {
+            bool ok = true;
+            for (int j = 0; j < 3 && ok; ++j) {
                 const int64_t pr = sq[j] >> 1;
-                if (!mbar_wait_cycles(smem_addr(&dfull[pr % kRowPairBufs]), (uint32_t)((pr / kRowPairBufs) & 1),
-                                      kTcWaitCycles)) {
-                    abort_flag = 1;
-                    return false;
-                }
+                ok = mbar_wait_cycles(smem_addr(&dfull[pr % kRowDone]), (uint32_t)((pr / kRowDone) & 1), kTcWaitCycles);
             }
-            if (abort_flag) return false;
+            // the warp goes on, or stops, as one: tcgen05.ld takes whole warps
+            if (!__all_sync(0xffffffffu, ok && !abort_flag)) {
+                abort_flag = 1;
+                return false;
+            }
             tc_fence_after();
             // the MMAs of input rows sq[0..2] are complete: free the input slot of
             // the last (each input row is some output row's sq[2], but for the
@@ -1021,13 +1034,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 
 }  // namespace
 
-// One 128-pixel column (W = 128) with more output rows than a wave of CTAs
-// (several rows per CTA, runs crossing image boundaries) is the shape of the
-// one GPU fault recorded for this library (CNN training at 32 x 128, batch 64;
-// Xid 13 and 43).  Reading the row-ring and weight-gradient kernels found no
-// out-of-range index for it, so the shape is kept off the tensor-core path:
-// the mma.sync kernels take it.  148 rows: at most one per CTA on a 148-SM or
-// larger part, the W = 128 shapes that run and are tested on this path.
+// One 128-pixel column (W = 128) with more output rows than a wave of CTAs is
+// kept off the tensor-core path: the mma.sync kernels take it.  32 x 128 inputs
+// at batch 64 once faulted in the row kernel, for the reason at kRowDone; that is
+// mended, but these shapes have not run on the row kernel since.  148 rows: at
+// most one per CTA on a 148-SM or larger part.
 constexpr int64_t kW128MaxRows = 148;
 
 bool w128_cleared(int B, int H, int W) { return W != 128 || (int64_t)B * H <= kW128MaxRows; }

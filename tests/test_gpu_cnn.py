@@ -96,6 +96,57 @@ def test_tensor_core_path_matches_mma_sync(L, H, W, B):
         L.cnn_destroy(m)
 
 
+def early_row_waits(B, H, W, barriers, sms=152):
+    """the row kernel's epilogue waits that a parity barrier lets pass too early:
+    pair p of accumulators on barrier p mod barriers, waited for by a warpgroup
+    that does not know pair p - barriers to be complete"""
+    rows = B * (W // 128) * H
+    early = 0
+    for cta in range(min(rows, sms)):
+        g0, g1 = rows * cta // min(rows, sms), rows * (cta + 1) // min(rows, sms)
+        known, n = [-1] * 4, 0
+        for k, g in enumerate(range(g0, g1)):
+            n += 3 if k == 0 or g % H == 0 else 1
+            for pair in ((n - 3) >> 1, (n - 2) >> 1, (n - 1) >> 1):
+                early += pair - barriers > known[k % 4]
+                known[k % 4] = max(known[k % 4], pair)
+    return early
+
+
+# shapes with CTAs whose first run of output rows has 1, 2 or 3 rows; at a height
+# of 8 with several runs in a CTA
+@pytest.mark.parametrize("H,W,B", [(64, 256, 14), (64, 256, 7), (32, 256, 23), (8, 256, 61), (8, 512, 30)])
+def test_row_kernel_waits_for_its_accumulators(L, H, W, B):
+    """A warpgroup's first output row may come after the end of the CTA's first
+    run.  With one barrier per accumulator pair (two) its wait passed before the
+    accumulators were written; with the ring of eight no wait does.  Against the
+    mma.sync path, with the bounds of the test above (targets of one sign, so
+    that the samples' gradients do not cancel)"""
+    assert early_row_waits(B, H, W, 2) > 0 and early_row_waits(B, H, W, 8) == 0
+    from oracle import cnn
+    xt, _ = inputs(B, H, W, 7)
+    y = torch.tensor(np.linspace(2, 3, B), dtype=torch.float32, device="cuda")
+    m = L.cnn_create(H, W, B, 3)
+    try:
+        assert L.cnn_tensor_core_paths(m, B) == (True, True)
+        out = []
+        for path in (1, 0):
+            L.cnn_set_conv_path(m, path)
+            pred, loss = (torch.zeros(n, dtype=torch.float32, device="cuda") for n in (B, 1))
+            L.cnn_forward(m, xt, pred)
+            L.cnn_gradient(m, xt, y, loss)
+            L.cnn_status(m)
+            out.append((pred.cpu().numpy().astype(np.float64), L.cnn_get_gradient(m).astype(np.float64)))
+        (p1, g1), (p0, g0) = out
+        assert np.abs(p0 - p1).max() <= 1e-2 * (np.abs(p1).max() + 1e-3)
+        off, _ = cnn.offsets()
+        for l in range(4):
+            sl = slice(off[l], off[l + 1])
+            assert np.linalg.norm(g0[sl] - g1[sl]) <= 2e-2 * np.linalg.norm(g1[sl]), l
+    finally:
+        L.cnn_destroy(m)
+
+
 def test_tensor_core_forward_at_full_size_matches_oracle(L, orc):
     """64 x 256 inputs (the 4x-downsampled 1024 x 256 channel), the shape the
     throughput bench runs: one row of 128 pixels per block, two blocks per row."""
