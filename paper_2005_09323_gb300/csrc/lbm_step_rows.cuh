@@ -90,7 +90,7 @@ __device__ __forceinline__ float rows_sites(const StepParams& p, const typename 
             }
         }
     }
-    if constexpr (V % 2 == 0 && S != kFP32) {
+    if constexpr (V % 2 == 0 && S != kFP32) {  // as in the register-staged step
         on_pairs(g, [&](auto& h, int i) { collide_pair<COLL>(h, i, p); });
     } else {
 #pragma unroll

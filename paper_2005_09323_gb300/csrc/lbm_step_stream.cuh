@@ -1,8 +1,8 @@
-// Two fused steps per pass over memory, for large ensembles of periodic channels
-// (App. A streaming and collision, twice): a block walks down the rows of a
-// channel, computes step t + 1 of row y + 1 and, from it and the two rows before,
-// step t + 2 of row y, so that a population value is read from HBM once and
-// written once for two steps.  A single step moves 72 bytes per site (FP32) and
+// Two fused steps per pass over memory, for large ensembles (App. A streaming and
+// collision, twice): a block walks down the rows of a channel, computes step t + 1
+// of row y + 1 and, from it and the two rows before, step t + 2 of row y, so that
+// a population value is read from HBM once and written once for two steps.  A
+// single step moves 72 bytes per site (FP32) and
 // is bound by HBM; here a site and step move 36 bytes.
 //
 // Thread = 4 consecutive sites, warp = 128 columns, block = a whole row, so the
@@ -31,8 +31,11 @@
 // latency.  Fewer registers and more warps spill and lose (FP16: 178 GLUPS at 128
 // registers, 171 at 102, 156 at 85).  Measured, single steps / streamed, GLUPS:
 // FP32 BGK 64 x 1024 x 256 94.6 / 158, 256 x 512 x 128 94.4 / 147, 16 x 2048 x 512
-// 93.3 / 160; FP32 central moments 93.6 / 123; FP16 BGK 157 / 185 (64 x 1024 x
-// 256), 159 / 203 (16 x 2048 x 512); FP16 central moments 132 / 138.
+// 93.3 / 160; FP32 central moments 93.6 / 123; FP16 BGK 163 / 184 (64 x 1024 x
+// 256), 164 / 201 (16 x 2048 x 512); FP16 central moments 142 / 149.  Open channels
+// of 513 x 129, 128 of them: FP32 central moments 70.6 / 83.9, FP32 BGK 75.6 / 79.9;
+// FP16 central moments 58.0 / 83.9; the work on their columns is a quarter to a
+// third of the streamed time.
 #pragma once
 #include "async_copy.cuh"
 #include "lbm_step.cuh"
@@ -118,17 +121,18 @@ __device__ __forceinline__ void stream_store(Vec<typename Codec<S>::T, kStreamV>
     }
 }
 
-// the collision of a thread's sites: BGK on pairs (161 against 150 GLUPS
-// without); the central-moment collision one site at a time, since on pairs its
+// the collision of a thread's sites, on pairs: BGK 161 against 150 GLUPS one site
+// at a time, FP16 central moments 149 against 137 (16 x 2048 x 512).  FP32
+// central moments in a periodic channel go one site at a time, since on pairs the
 // constants and temporaries take registers the row loop does not have (96 bytes
-// of spills, 126 against 127 GLUPS at 64 x 1024 x 256, 123 against 134 at 256 x 512 x 128)
-// An open channel's sites relax at their columns' rates om.
-template <int COLL, bool OPEN>
+// of spills, 126 against 127 GLUPS at 64 x 1024 x 256, 123 against 134 at 256 x 512 x
+// 128).  An open channel's sites relax at their columns' rates om.
+template <int S, int COLL, bool OPEN>
 __device__ __forceinline__ void stream_collide(float2 (&g)[9][kStreamV / 2], const StepParams& p,
                                                const float2 (&om)[kStreamV / 2])
 {
-    if constexpr (COLL == 0 && !OPEN) {
-        collide2<0, kStreamV / 2>(g, p);
+    if constexpr ((COLL == 0 || S != kFP32) && !OPEN) {
+        collide2<COLL, kStreamV / 2>(g, p);
     } else if constexpr (OPEN) {
 #pragma unroll
         for (int i = 0; i < kStreamV / 2; ++i) collide_at2<COLL>(g, i, p, om[i]);
@@ -291,7 +295,7 @@ __device__ __forceinline__ float stream_site_group(const StepParams& p, float2 (
     if constexpr (OPEN) {
         float2 om[V / 2];
         stream_rates(p, x, om);
-        stream_collide<COLL, true>(g, p, om);
+        stream_collide<S, COLL, true>(g, p, om);
     } else {
         collide2<COLL, V / 2>(g, p);
     }
@@ -721,7 +725,7 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
             om[0] = make_float2(o.x, o.y);
             om[1] = make_float2(o.z, o.w);
         }
-        stream_collide<COLL, OPEN>(g, p, om);
+        stream_collide<S, COLL, OPEN>(g, p, om);
     };
 
     if (tid < 4 * nwarp) mbar_init(smem_addr(&edge_ready[tid & 3][tid >> 2]), 1);
