@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cmath>
 #include <limits>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -81,10 +82,40 @@ __global__ void drag_square_kernel(const double* drag, int32_t max_steps, int32_
 // clock and SM on this GPU, 1.2 ms for the 7e8 products of 64 x 6500 steps and
 // 2000 lags; 32-bit integer multiply-adds with 64-bit sums run 32 times as many.
 // A fluctuation x is rounded to X = x 2^k with the largest below 2^54 (an error
-// of 2^-55 of the largest, below the 2^-53 of an FP64 fluctuation) and split
-// into X = hi 2^28 + lo, |hi| <= 2^26 + 1, |lo| <= 2^27.  Every product and every
-// sum after that is exact, so the result does not depend on their order.
+// of 2^-55 of the largest, below the 2^-53 of an FP64 fluctuation of that size) and split
+// into X = hi 2^28 + lo, |hi| <= 2^26 + 1, |lo| <= 2^27.  Every product is exact, and so
+// is every sum after that, so the result does not depend on their order: 128
+// bits would hold 2^19 products of the largest value (128 sine series of 20000
+// steps sum to 2.2 x 2^127), so longer sums are kept in 160 bits, which hold 2^51.
 constexpr int kLimb = 28;
+
+// a sum of 128-bit integers v as that of v >> 32 and that of their low 32 bits
+struct WideSum {
+    __int128 high = 0;
+    unsigned long long low = 0;
+    __device__ void add(__int128 v)
+    {
+        high += v >> 32;
+        low += (unsigned int)v;
+    }
+    __device__ void add(__int128 h, unsigned long long l)
+    {
+        high += h;
+        low += l;
+    }
+    __device__ double value() const
+    {
+        __int128 h = high + (long long)(low >> 32);
+        long long l = (long long)(low & 0xffffffffull);
+        const bool negative = h < 0;  // then h 2^32 + l < 0: of the magnitude, no digits cancel
+        if (negative) {
+            h = -h;
+            l = -l;
+        }
+        const double v = ((double)(long long)(h >> 64) * 0x1.0p64 + (double)(unsigned long long)h) * 0x1.0p32 + (double)l;
+        return negative ? -v : v;
+    }
+};
 
 // k of the quantisation; 0 for an all-zero or a non-finite series
 __device__ int fixed_exponent(const double* stat, int32_t n, double* sh)
@@ -124,19 +155,42 @@ __global__ void drag_limbs_kernel(const double* drag, int32_t max_steps, int32_t
 // and takes four times t at once from registers (16 products, 48 multiply-adds,
 // for six 16-byte shared-memory loads; three multiply-adds a product instead of
 // four through (hi + lo)(hi' + lo') - hi hi' - lo lo').  A block takes kCorrLags lags and walks
-// its share of the (clone, kCorrTime steps) tasks; partial[split][lag].
-constexpr int kCorrThreads = 128, kCorrLags = 4 * kCorrThreads, kCorrTime = 512, kCorrFlush = 128;
+// its share of the (clone, kCorrTime steps) tasks; partial[split][lag].  A thread
+// sums kCorrTasks tasks, 2^18 products, in 128 bits.  WIDE: it has more, and adds
+// each kCorrTasks of them to its sum's halves in partial and low (the plain form
+// stays beside it for its registers: 286 against 297 us, 64 x 6500 and 2000 lags).
+constexpr int kCorrThreads = 128, kCorrLags = 4 * kCorrThreads, kCorrTime = 512, kCorrFlush = 128, kCorrTasks = 512;
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kCorrThreads) autocorr_kernel(const int32_t* hi, const int32_t* lo, int32_t n,
                                                                 int32_t len, int32_t pitch, int32_t n_lags,
-                                                                __int128* partial)
+                                                                __int128* partial, unsigned long long* low)
 {
     constexpr int kWin = kCorrTime + kCorrLags + 4;
     __shared__ __align__(16) int32_t ah[kCorrTime], al[kCorrTime], as[kCorrTime], bh[kWin], bl[kWin], bs[kWin];
     const int chunks = (len + kCorrTime - 1) / kCorrTime, tasks = n * chunks;
     const int lag0 = blockIdx.x * kCorrLags, l0 = 4 * threadIdx.x;
     __int128 sum[4] = {0, 0, 0, 0};
+    auto store = [&](bool more) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (lag0 + l0 + j >= n_lags) continue;
+            const int64_t i = (int64_t)blockIdx.y * n_lags + lag0 + l0 + j;
+            if constexpr (WIDE) {
+                WideSum w;
+                if (more) w.add(partial[i], low[i]);
+                w.add(sum[j]);
+                partial[i] = w.high;
+                low[i] = w.low;
+                sum[j] = 0;
+            } else {
+                partial[i] = sum[j];
+            }
+        }
+    };
+    int done = 0;
     for (int task = blockIdx.y; task < tasks; task += gridDim.y) {
+        if (WIDE && done++ % kCorrTasks == 0 && done > 1) store(done > kCorrTasks + 1);
         const int c = task / chunks, tb = (task - c * chunks) * kCorrTime;
         if (tb + lag0 >= len) continue;  // block-uniform: every product is past the series
         const int32_t *rh = hi + (int64_t)c * pitch, *rl = lo + (int64_t)c * pitch;
@@ -180,29 +234,39 @@ __global__ void __launch_bounds__(kCorrThreads) autocorr_kernel(const int32_t* h
                 sum[j] += ((__int128)hh[j] << (2 * kLimb)) + (((__int128)ss[j] - hh[j] - ll[j]) << kLimb) + (__int128)ll[j];
         }
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (lag0 + l0 + j < n_lags) partial[(int64_t)blockIdx.y * n_lags + lag0 + l0 + j] = sum[j];
+    store(done > kCorrTasks);
 }
 
 // C(lag) = sum of products / their number / variance; the first lag with C <= 0.
 // A block takes 32 lags, each of its warps a part of the splits.
-__global__ void __launch_bounds__(kStatThreads) autocorr_final_kernel(const __int128* partial, int32_t splits, int32_t n_lags, const double* stat,
-                                      int32_t n, int32_t len, double* c, int32_t* first)
+template <bool WIDE>
+__global__ void __launch_bounds__(kStatThreads) autocorr_final_kernel(const __int128* partial,
+                                                                      const unsigned long long* low, int32_t splits,
+                                                                      int32_t n_lags, const double* stat, int32_t n,
+                                                                      int32_t len, double* c, int32_t* first)
 {
     __shared__ double sh[kStatThreads];
     const double var = sum_over(stat + n, n, sh) / ((double)n * (double)len);
     const int k = fixed_exponent(stat, n, sh);
-    __shared__ __int128 part[kStatThreads / 32][32];
+    __shared__ __int128 part_h[kStatThreads / 32][32];
+    __shared__ unsigned long long part_l[kStatThreads / 32][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lag = blockIdx.x * 32 + lane;
-    __int128 s = 0;
+    WideSum s;
     if (lag < n_lags)
-        for (int i = warp; i < splits; i += kStatThreads / 32) s += partial[(int64_t)i * n_lags + lag];
-    part[warp][lane] = s;
+#pragma unroll 4
+        for (int i = warp; i < splits; i += kStatThreads / 32) {
+            const int64_t at = (int64_t)i * n_lags + lag;
+            if constexpr (WIDE)
+                s.add(partial[at], low[at]);
+            else
+                s.add(partial[at]);
+        }
+    part_h[warp][lane] = s.high;
+    part_l[warp][lane] = s.low;
     __syncthreads();
     if (warp != 0 || lag >= n_lags) return;
-    for (int w = 1; w < kStatThreads / 32; ++w) s += part[w][lane];
-    const double x = scalbn(scalbn((double)(long long)(s >> 64) * 0x1.0p64 + (double)(unsigned long long)s, -k), -k);
+    for (int w = 1; w < kStatThreads / 32; ++w) s.add(part_h[w][lane], part_l[w][lane]);
+    const double x = scalbn(scalbn(s.value(), -k), -k);
     const double v = x / ((double)n * (double)(len - lag)) / var;
     c[lag] = v;
     if (v <= 0.0) atomicMin(first, lag);
@@ -312,11 +376,16 @@ int lbm_drag_autocorrelation(lbm_ensemble* e, int32_t t0, int32_t t1, int32_t ma
     if (tasks > INT32_MAX) return fail(LBM_ERR_ARG, "lbm_drag_autocorrelation: series too long");
     const int splits = (int)std::min<int64_t>(tasks, std::max(1, 152 * 12 / lag_tiles));
     const size_t limb_bytes = sizeof(int32_t) * (size_t)n * pitch, stat_bytes = (sizeof(double) * 3 * n + 15) / 16 * 16;
+    const size_t sums = (size_t)splits * lags;
+    const bool wide = (tasks + splits - 1) / splits > kCorrTasks;
     Workspace ws;
-    if (int rc = stat_workspace(e, 16 + sizeof(__int128) * (size_t)splits * lags + stat_bytes + 2 * limb_bytes, &ws)) return rc;
+    if (int rc = stat_workspace(e, 16 + sizeof(__int128) * sums + (wide ? sizeof(long long) * sums : 0) + stat_bytes +
+                                       2 * limb_bytes, &ws)) return rc;
     int32_t* first = reinterpret_cast<int32_t*>(ws.p);
     __int128* partial = reinterpret_cast<__int128*>(ws.p + 16);
-    double* stat = reinterpret_cast<double*>(ws.p + 16 + sizeof(__int128) * (size_t)splits * lags);
+    double* stat = reinterpret_cast<double*>(partial + sums);
+    unsigned long long* low = reinterpret_cast<unsigned long long*>(ws.p + 16 + sizeof(__int128) * sums + stat_bytes +
+                                                                    2 * limb_bytes);
     int32_t* hi = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(stat) + stat_bytes);
     int32_t* lo = hi + (size_t)n * pitch;
     LBM_CUDA(cudaMemsetAsync(first, 0x7f, sizeof(int32_t), e->stream));
@@ -324,9 +393,17 @@ int lbm_drag_autocorrelation(lbm_ensemble* e, int32_t t0, int32_t t1, int32_t ma
     drag_square_kernel<<<n, kStatThreads, 0, e->stream>>>(e->drag, e->cfg.max_steps, n, t0, len, stat);
     drag_limbs_kernel<<<dim3((pitch + kStatThreads - 1) / kStatThreads, n), kStatThreads, 0, e->stream>>>(
         e->drag, e->cfg.max_steps, n, t0, len, stat, pitch, hi, lo);
-    autocorr_kernel<<<dim3(lag_tiles, splits), kCorrThreads, 0, e->stream>>>(hi, lo, n, len, pitch, lags, partial);
-    autocorr_final_kernel<<<(lags + 31) / 32, kStatThreads, 0, e->stream>>>(
-        partial, splits, lags, stat, n, len, c_dev, first);
+    auto correlate = [&](auto w) {
+        constexpr bool WIDE = decltype(w)::value;
+        autocorr_kernel<WIDE><<<dim3(lag_tiles, splits), kCorrThreads, 0, e->stream>>>(hi, lo, n, len, pitch, lags,
+                                                                                     partial, low);
+        autocorr_final_kernel<WIDE><<<(lags + 31) / 32, kStatThreads, 0, e->stream>>>(partial, low, splits, lags, stat,
+                                                                                   n, len, c_dev, first);
+    };
+    if (wide)
+        correlate(std::true_type{});
+    else
+        correlate(std::false_type{});
     LBM_CUDA(cudaGetLastError());
     count_launches(5);
     if (tau_c) {
