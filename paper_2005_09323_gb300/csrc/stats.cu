@@ -319,24 +319,34 @@ __global__ void __launch_bounds__(32 * kUpWarps) upcross_kernel(const double* dr
 }
 
 // A workspace of at least `bytes` for one call: the ensemble's own, grown on
-// demand and kept until the ensemble is destroyed (used in its stream's order),
-// or, where it would have to grow while the stream is being captured, an
-// allocation of the captured work itself (temporary: released by the caller).
+// demand and kept until the ensemble is destroyed (used in its stream's order).
+// A call that is being captured takes an allocation of the captured work itself
+// instead, released behind it on every way out: the ensemble's own may have been
+// replaced by a larger one when the captured work is replayed.
 struct Workspace {
     char* p = nullptr;
+    cudaStream_t captured = nullptr;
     bool temporary = false;
+    Workspace() = default;
+    Workspace(const Workspace&) = delete;
+    Workspace& operator=(const Workspace&) = delete;
+    ~Workspace()
+    {
+        if (temporary) cudaFreeAsync(p, captured);
+    }
 };
 
 int stat_workspace(lbm_ensemble* e, size_t bytes, Workspace* ws)
 {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    LBM_CUDA(cudaStreamIsCapturing(e->stream, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone) {
+        LBM_CUDA(cudaMallocAsync((void**)&ws->p, bytes, e->stream));
+        ws->captured = e->stream;
+        ws->temporary = true;
+        return LBM_OK;
+    }
     if (e->stat_bytes < bytes) {
-        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-        LBM_CUDA(cudaStreamIsCapturing(e->stream, &capturing));
-        if (capturing != cudaStreamCaptureStatusNone) {
-            LBM_CUDA(cudaMallocAsync((void**)&ws->p, bytes, e->stream));
-            ws->temporary = true;
-            return LBM_OK;
-        }
         LBM_CUDA(cudaStreamSynchronize(e->stream));
         if (e->stat_ws) cudaFree(e->stat_ws);
         e->stat_ws = nullptr;
@@ -411,7 +421,6 @@ int lbm_drag_autocorrelation(lbm_ensemble* e, int32_t t0, int32_t t1, int32_t ma
         LBM_CUDA(cudaStreamSynchronize(e->stream));
         if (*tau_c > max_lag) *tau_c = -1;
     }
-    if (ws.temporary) LBM_CUDA(cudaFreeAsync(ws.p, e->stream));
     return LBM_OK;
 }
 

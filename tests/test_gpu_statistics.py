@@ -80,3 +80,37 @@ def test_autocorrelation_at_tile_edges(L, n, steps, t0, max_lag):
         c = torch.zeros(max_lag + 1, dtype=torch.float64, device="cuda")
         L.lbm_drag_autocorrelation(e, t0, steps, max_lag, c)
     assert np.allclose(c.cpu().numpy()[lags], reference(d[:, t0:], lags), rtol=1e-10, atol=1e-12)
+
+
+def test_captured_autocorrelation_outlives_the_workspace(L):
+    """A call captured after a warm-up, then a larger call that replaces the
+    ensemble's workspace, then the captured work replayed on a changed series:
+    the same bits as a direct call, and the larger call's result untouched"""
+    rng = np.random.default_rng(3)
+    n, steps, lag = 4, 3000, 40
+    d = rng.normal(0.4, 0.01, (n, steps))
+    s = torch.cuda.Stream()
+    with Series(L, d, s) as e:
+        small, direct = (torch.zeros(lag + 1, dtype=torch.float64, device="cuda") for _ in range(2))
+        large = torch.zeros(2900, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        call = L.lib().lbm_drag_autocorrelation
+        assert call(e, 0, 600, lag, small.data_ptr(), None) == 0
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            assert call(e, 0, 600, lag, small.data_ptr(), None) == 0
+        L.lbm_drag_autocorrelation(e, 0, steps, 2899, large)
+        before = large.clone()
+        d[:, :600] = rng.normal(0.4, 0.02, (n, 600))
+        L.lbm_ensemble_set_drag(e, 0, steps, d)
+        small.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            for _ in range(2):
+                g.replay()
+        s.synchronize()
+        L.lbm_drag_autocorrelation(e, 0, 600, lag, direct)
+        assert torch.equal(small, direct) and float(direct[0]) != 0.0
+        assert torch.equal(large, before)
+        del g
