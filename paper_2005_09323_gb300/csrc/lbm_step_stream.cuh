@@ -866,6 +866,7 @@ __global__ void __launch_bounds__(kStreamMaxThreads, 1) step_stream_kernel(const
                 C4 = ws.up[(k + 1) & 1][0][lane];
                 C7 = ws.up[(k + 1) & 1][1][lane];
                 C8 = ws.up[(k + 1) & 1][2][lane];
+                __syncwarp();  // every lane has read the edge values of the rows before
             }
             const VT A2 = ws.up[k & 1][0][lane], A5 = ws.up[k & 1][1][lane], A6 = ws.up[k & 1][2][lane];
             if (real) {
