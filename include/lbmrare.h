@@ -241,7 +241,9 @@ int lbm_ensemble_set_observables(lbm_ensemble* e, int32_t enable);
 int lbm_ensemble_observables(lbm_ensemble* e, int32_t t0, int32_t t1, double* dst, int32_t dst_on_device);
 
 /* Fluid mass and momentum sum_x sum_q f_q (1, c_q) per clone (host double[N]
- * each; any may be NULL), FP64 deterministic reduction.  Waits. */
+ * each; any may be NULL), deterministic: per thread compensated FP32 pairs, which
+ * hold the sums of stored populations exactly (FP64 where one leaves FP32's range),
+ * then FP64 in a fixed order.  Waits. */
 int lbm_ensemble_moments(lbm_ensemble* e, double* mass, double* px, double* py);
 
 /* Read / overwrite one clone's populations as FP64 [9][ny][nx] host arrays
@@ -319,7 +321,14 @@ int lbm_ensemble_kernel_time(lbm_ensemble* e, double* ms, int64_t* launches, int
 
 /* Drag statistics of direct sampling.  The clones are independent
  * trajectories; their drag series over the steps [t0, t1) are pooled (every
- * clone must have reached t1).  FP64, every sum in a fixed order.
+ * clone must have reached t1).  Mean and variance are FP64 sums in a fixed order;
+ * the products of the autocorrelation are exact integers, the fluctuations
+ * rounded to 2^-55 of the largest one.  Neither result depends on timing.  The
+ * calls keep a workspace until the ensemble is destroyed, up to 8 bytes per clone
+ * and step of the window (rounded up to 512 steps) and 16 bytes (24 on series of
+ * 10^8 values and more) per lag and partial sum; one that needs a larger workspace
+ * waits and allocates it.  While the stream is being captured a call allocates its
+ * workspace in the captured work instead.
  *
  * lbm_drag_autocorrelation: c_dev[tau] (device, max_lag + 1 doubles) =
  *   mean_{clones, t} f~(t + tau) f~(t) / mean f~^2,   f~ = f_d - mean f_d,
