@@ -950,6 +950,32 @@ inline int stream_threads(const StepParams& p)
     return ((p.open ? p.nx - 1 : p.nx) + 32 * kStreamV - 1) / (32 * kStreamV) * 32;
 }
 
+// blocks an SM holds: of the 512 threads that 128 registers leave room for, those
+// that fit its shared memory.  FP32 rows of at most 128 sites: 15 blocks of a warp, not
+// 16; a grid of 16 an SM left 152 blocks to a second wave (128 x 64, 494 clones,
+// us a step with 16 / 15: BGK 36.4 / 32.4, central moments 50.3 / 42.1)
+template <int S>
+int stream_blocks_per_sm(int threads)
+{
+    constexpr int kStatic = 4 * 6 * (kStreamMaxThreads / 32) * (int)sizeof(typename Codec<S>::T) +
+                            4 * (kStreamMaxThreads / 32) * (int)sizeof(uint64_t);
+    int dev = 0, smem = 228 * 1024, reserved = 1024;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    }
+    const int bytes = threads / 32 * (int)sizeof(StreamWarpSmem<S>) + kStatic + reserved;
+    const int fit = smem / ((bytes + 127) / 128 * 128), most = kStreamMaxThreads / threads;
+    return fit < 1 ? 1 : (fit < most ? fit : most);
+}
+
+inline int stream_sms()
+{
+    int sms = 152, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 // whole rows of at most 2048 sites in a block, the work apart in its shared
 // memory; in an open channel the column ranges and the obstacle's region apart
 template <int S>
@@ -971,10 +997,8 @@ template <int S, bool SCALED, int COLL, bool OPEN>
 cudaError_t launch_stream_kernel(const StepParams& p, cudaStream_t s)
 {
     const int threads = stream_threads(p);
-    const int ctas = kStreamMaxThreads / threads;  // per SM: the 512 threads that 128 registers leave room for
+    const int ctas = stream_blocks_per_sm<S>(threads), sms = stream_sms();
     const size_t smem = threads / 32 * sizeof(StreamWarpSmem<S>);
-    int sms = 152, dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t rows = (int64_t)p.n_list * p.ny;
     const int grid = (int)(rows < (int64_t)ctas * sms ? rows : (int64_t)ctas * sms);
     const cudaError_t e = cudaFuncSetAttribute(step_stream_kernel<S, SCALED, COLL, OPEN>,

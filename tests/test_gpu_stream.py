@@ -110,3 +110,13 @@ def test_default_streams_large_calls_only(L):
         assert L.lbm_launch_count() - l0 == 8 + 8 + 1
     finally:
         L.lbm_ensemble_destroy(e)
+
+
+@pytest.mark.parametrize("nx", [64, 128])
+def test_one_warp_rows_over_more_rows_than_blocks(L, nx):
+    """rows of one warp, 15 (FP32) or 16 blocks an SM: spans of one, two and several
+    rows, over clone boundaries"""
+    for storage, n in (("fp32", 150), ("fp32", 290), ("fp16", 700)):
+        cfg = L.config(nx, 16, obstacle=(20, 6, 5, 5), tau=0.56, gx=2e-6, storage=storage, max_steps=16)
+        a, b = (run(L, cfg, n, (8,), variant(L, storage, k)) for k in (0, 3))
+        assert np.array_equal(a[0], b[0]) and all(np.array_equal(x, y) for x, y in zip(a[1], b[1])), (storage, n)
