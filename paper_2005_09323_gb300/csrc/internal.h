@@ -37,6 +37,7 @@ struct StepVariant {
     // variant has no open-channel instantiation
     Launch launch_open = nullptr;
     int multi = 1;  // most steps one launch runs (kind 2: an odd number per launch; kind 3: one or two)
+    bool (*pays)(const StepParams&) = nullptr;  // kind 3: faster than single steps of the default variant
 };
 
 // LBM_ERR_ARG unless the collision fields of c are valid (lbm_ensemble.cu)

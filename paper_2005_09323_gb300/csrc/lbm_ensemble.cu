@@ -770,13 +770,7 @@ int stream_variant(int storage)
 }
 
 // the variant of a step call over n_list clones.  A call of four steps and more
-// streams rows, two steps per pass over memory, if every
-// block then has enough rows: a block recomputes two rows of its span, and each
-// of its rows waits on the one before.  Measured on channels of 128 to 2048
-// columns (single steps / streamed, us per step): FP32 BGK 16.6 / 17.1 at 5
-// rows a block, 23.1 / 19.9 at 7, 37.0 / 26.1 at 10, 178 / 105 at 54; FP32
-// central moments 24.6 / 26.0 at 7, 36.9 / 33.3 at 10; FP16 BGK 14.9 / 15.6 at
-// 7, 24.2 / 20.3 at 10; FP16 central moments 30.2 / 30.7 at 10, 39.2 / 36.8 at 13.
+// streams rows, two steps per pass over memory, where that pays (stream_pays)
 int variant_for(const lbm_ensemble* e, int n_list, int n_steps)
 {
     const lbm_config& c = e->cfg;
@@ -788,18 +782,8 @@ int variant_for(const lbm_ensemble* e, int n_list, int n_steps)
     if (e->variant_tuned && vi != s) return vi;
     vi = e->variant_tuned ? default_variant(c.storage) : vi;
     if (e->observe || n_steps < 4 || s < 0) return vi;
-    if (!vars[s].supports(make_params(e, e->all_dev, n_list, vars[s].vec, 0, 3))) return vi;
-    const int threads = ((c.open_x ? c.nx - 1 : c.nx) + 127) / 128 * 32;
-    const int64_t blocks = (int64_t)(512 / threads) * 152;
-    // (open channels, 513 x 129, the work on their columns included: FP32 central
-    // moments 32.0 / 36.8 us at 7 rows a block, 61.4 / 57.8 at 14; FP32 BGK 57.3 /
-    // 61.4 at 14, 113 / 109 at 27; FP16 central moments 18.9 / 21.3 at 3, 38.1 /
-    // 28.4 at 7, 74.4 / 52.3 at 14; FP16 BGK 35.4 / 25.5 at 7)
-    const int64_t min_rows = !c.open_x                ? (c.collision == 0 ? 8 : 12)
-                             : c.storage != LBM_FP32 ? 6
-                             : c.collision == 1      ? 12
-                                                     : 24;
-    return (int64_t)n_list * c.ny >= min_rows * blocks ? s : vi;
+    const StepParams p = make_params(e, e->all_dev, n_list, vars[s].vec, 0, 3);
+    return vars[s].supports(p) && vars[s].pays(p) ? s : vi;
 }
 
 int check_sticky(lbm_ensemble* e)

@@ -993,6 +993,53 @@ bool stream_supported(const StepParams& p)
     return true;
 }
 
+// whether calls of four steps and more take less time streamed than in single steps
+// of the default variant.  In units of a streamed row's time, with R rows a block, a
+// block takes R + 2 of them (it recomputes two), c for every row's worth of sites
+// computed apart, and d shared by the SM's blocks, whose apart work and first rows
+// overlap with the others' rows; single steps take `gain` rows for each row.  16-bit
+// steps are bound by instructions: there the lanes that the single step's 256-column
+// segments leave idle count, and the warps that the SM lacks where rows of 5, 6 or 7
+// warps leave some out.  The figures are fitted to 952 measurements, single and
+// streamed, channels of 64 to 2049 columns, 4 to 48 rows a block, obstacles up to 3/4
+// and grids up to 64 columns wide; the choice costs 0.4 % on average, at most 10 %
+// (16-bit rows of 640 and 2049 columns), 17 % where it stays with single steps.
+// Some (us a step, single / streamed):
+//   FP32 BGK      1024 x 256, 32 x 32 square, 15 clones 45.8 / 29.9; with 200 x 200 48.3 / 49.5
+//   FP32 CM       1024 x 256, 15 clones 45.4 / 38.9; 200 x 200, 48 clones 151 / 176
+//   FP16 BGK      2048 x 512, 12 clones 78.7 / 66.1; 256 x 64, 32 x 32, 247 clones 36.2 / 45.8
+//   FP16 CM       2048 x 512, 12 clones 90.1 / 88.5; 512 x 128, 64 x 64, 190 clones 107 / 129
+//   open FP32 CM  513 x 129, 61 clones 58.9 / 56.4; 2049 x 513, 4 clones 52.9 / 61.4
+//   open FP32 BGK 513 x 129, 118 clones 104 / 98.9; bars of 64 columns, 127 clones 114 / 124
+//   open FP16 CM  513 x 129, 66 clones 76.5 / 54.7; 769 x 193, 22 clones 40.8 / 48.2
+template <int S>
+bool stream_pays(const StepParams& p)
+{
+    constexpr int G = kStreamGroup<S>;
+    const int threads = stream_threads(p), ctas = stream_blocks_per_sm<S>(threads);
+    const double rows = (double)p.n_list * p.ny / ((double)ctas * stream_sms());
+    const StreamRegion<S> rg(p);
+    double apart = (double)rg.ng * G * (rg.r1 - rg.r0) / ((double)p.nx * p.ny);
+    if (p.open) {
+        const StreamColumns<S> cols(p);
+        for (int r = 0; r < 3; ++r)
+            if (cols.g1[r] > cols.g0[r]) apart += (double)(cols.g1[r] - cols.g0[r]) * G / p.nx;
+    }
+    struct Cost {
+        double gain, c, d;
+    };
+    const bool bgk = p.coll == 0;
+    const Cost k = S == kFP32 ? (p.open ? (bgk ? Cost{1.6, 3.0, 20.0} : Cost{1.8, 1.0, 20.0})
+                                        : (bgk ? Cost{1.5, 3.0, 1.0} : Cost{1.35, 3.0, 1.0}))
+                              : (p.open ? Cost{2.2, 0.0, 20.0} : (bgk ? Cost{1.6, 8.0, 9.0} : Cost{1.1, 2.0, 1.0}));
+    double gain = k.gain;
+    if (S != kFP32) {
+        const int segments = ((p.open ? p.nx - 1 : p.nx) + 32 * G - 1) / (32 * G);
+        gain *= (double)segments * 32 * G / (threads * kStreamV) * (ctas * threads) / kStreamMaxThreads;
+    }
+    return rows * (gain - 1.0 - k.c * apart) >= 2.0 + k.d / ctas;
+}
+
 template <int S, bool SCALED, int COLL, bool OPEN>
 cudaError_t launch_stream_kernel(const StepParams& p, cudaStream_t s)
 {

@@ -22,6 +22,7 @@ void register_step_bf16(std::vector<StepVariant>& out)
     // two steps per pass over memory: large ensembles
     out.push_back({kBF16, kStreamGroup<kBF16>, kStreamMaxThreads / 32, &launch_stream<kBF16>, 3, &stream_supported<kBF16>});
     out.back().multi = 2;
+    out.back().pays = &stream_pays<kBF16>;
 }
 
 }  // namespace lbm

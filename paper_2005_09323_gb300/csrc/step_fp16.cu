@@ -22,6 +22,7 @@ void register_step_fp16(std::vector<StepVariant>& out)
     // two steps per pass over memory: large ensembles
     out.push_back({kFP16, kStreamGroup<kFP16>, kStreamMaxThreads / 32, &launch_stream<kFP16>, 3, &stream_supported<kFP16>});
     out.back().multi = 2;
+    out.back().pays = &stream_pays<kFP16>;
 }
 
 }  // namespace lbm

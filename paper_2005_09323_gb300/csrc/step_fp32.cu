@@ -36,6 +36,7 @@ void register_step_fp32(std::vector<StepVariant>& out)
     // two steps per pass over memory: large ensembles
     out.push_back({kFP32, kStreamGroup<kFP32>, kStreamMaxThreads / 32, &launch_stream<kFP32>, 3, &stream_supported<kFP32>});
     out.back().multi = 2;
+    out.back().pays = &stream_pays<kFP32>;
 }
 
 }  // namespace lbm

@@ -120,3 +120,34 @@ def test_one_warp_rows_over_more_rows_than_blocks(L, nx):
         cfg = L.config(nx, 16, obstacle=(20, 6, 5, 5), tau=0.56, gx=2e-6, storage=storage, max_steps=16)
         a, b = (run(L, cfg, n, (8,), variant(L, storage, k)) for k in (0, 3))
         assert np.array_equal(a[0], b[0]) and all(np.array_equal(x, y) for x, y in zip(a[1], b[1])), (storage, n)
+
+
+OPEN_KW = dict(open_x=1, u_in=0.05, sponge_tau=1.0, collision="cm", tau=0.53)
+
+
+@pytest.mark.parametrize("n,nx,ny,storage,kw,streams", [
+    # measured slower streamed: large squares, few 16-bit rows, wide rows with few rows a
+    # block, wide grids
+    (15, 1024, 256, "fp32", dict(obstacle=(158, 28, 200, 200)), False),
+    (48, 1024, 256, "fp32", dict(obstacle=(158, 28, 200, 200), collision="cm"), False),
+    (190, 512, 128, "fp16", dict(obstacle=(98, 32, 64, 64)), False),
+    (247, 256, 64, "bf16", dict(obstacle=(50, 16, 32, 32)), False),
+    (4, 2049, 513, "fp32", dict(OPEN_KW, obstacle=(992, 224, 64, 64), grid=(64, 32, 32, 32), sponge_len=512), False),
+    (4, 2049, 513, "fp16", dict(OPEN_KW, obstacle=(992, 224, 64, 64), grid=(64, 32, 32, 32), sponge_len=512), False),
+    (127, 513, 129, "fp32", dict(OPEN_KW, collision="bgk", obstacle=(248, 56, 16, 16), grid=(16, 64, 8, 8),
+                                 sponge_len=128), False),
+    # measured faster streamed
+    (64, 1024, 256, "fp32", dict(obstacle=(240, 112, 32, 32)), True),
+    (16, 2048, 512, "fp16", dict(obstacle=(480, 224, 64, 64)), True),
+    (64, 513, 129, "fp32", dict(OPEN_KW, obstacle=(248, 56, 16, 16), grid=(16, 8, 8, 8), sponge_len=128), True),
+    (64, 513, 129, "bf16", dict(OPEN_KW, obstacle=(248, 56, 16, 16), grid=(16, 8, 8, 8), sponge_len=128), True),
+    (494, 128, 64, "fp32", dict(obstacle=(32, 29, 6, 6), collision="cm"), True),
+])
+def test_default_streams_where_it_pays(L, n, nx, ny, storage, kw, streams):
+    """eight steps: four launches streamed, eight single ones otherwise, and the drag's
+    (the open channel's single steps also launch its outlet)"""
+    cfg = L.config(nx, ny, max_steps=16, storage=storage, **dict(dict(tau=0.53), **kw))
+    drag, pops, launches = run(L, cfg, n, (8,))
+    assert launches == (5 if streams else 9 + (1 if kw.get("open_x") else 0))
+    ref = run(L, cfg, n, (8,), variant(L, storage, 0))
+    assert np.array_equal(drag, ref[0]) and all(np.array_equal(x, y) for x, y in zip(pops, ref[1]))
