@@ -284,7 +284,8 @@ int lbm_ensemble_autotune(lbm_ensemble* e, int32_t* variant);
  * sites (clones x nx x ny, e.g. one AMS branch) use a separate small-list
  * variant (default: the narrowest register-staged variant with 8 warps, which
  * puts the most threads on a small grid); lbm_ensemble_autotune picks both.
- * Step calls of four steps and more over many rows stream rows, two steps per pass over memory, unless a variant is forced; the
+ * Step calls of four steps and more over many rows stream rows, two steps per
+ * pass over memory, unless a variant is forced or another one tuned; the
  * populations and the drag are the default variant's bit for bit. */
 int lbm_ensemble_set_variant(lbm_ensemble* e, int32_t variant);
 int lbm_step_variant_info(int32_t variant, int32_t* storage, int32_t* vec, int32_t* warps);

@@ -133,6 +133,7 @@ struct lbm_ensemble {
     // calls over many sites, one for calls below kSmallSites (an AMS branch)
     int variant;
     int variant_small;
+    int variant_single;       // tuned: of the calls that do not stream rows, when `variant` does
     bool variant_forced;      // by lbm_ensemble_set_variant: runs every call
     bool variant_tuned;       // by lbm_ensemble_autotune
     // step chunks captured once as CUDA graphs and replayed: one cached

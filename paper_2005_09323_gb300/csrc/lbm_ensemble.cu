@@ -770,20 +770,20 @@ int stream_variant(int storage)
 }
 
 // the variant of a step call over n_list clones.  A call of four steps and more
-// streams rows, two steps per pass over memory, where that pays (stream_pays)
+// streams rows, two steps per pass over memory, where that pays (stream_pays) or, over
+// all clones, where lbm_ensemble_autotune measured it as the fastest.  What does not
+// stream runs the tuned single-step variant, else the default one
 int variant_for(const lbm_ensemble* e, int n_list, int n_steps)
 {
     const lbm_config& c = e->cfg;
     if ((int64_t)n_list * c.nx * c.ny <= kSmallSites) return e->variant_small;
     const auto& vars = step_variants();
-    int vi = e->variant;
-    if (e->variant_forced) return vi;
     const int s = stream_variant(c.storage);
-    if (e->variant_tuned && vi != s) return vi;
-    vi = e->variant_tuned ? default_variant(c.storage) : vi;
-    if (e->observe || n_steps < 4 || s < 0) return vi;
+    if (e->variant_forced || (e->variant_tuned && e->variant != s)) return e->variant;
+    const int single = e->variant_tuned ? e->variant_single : e->variant;
+    if (e->observe || n_steps < 4 || s < 0) return single;
     const StepParams p = make_params(e, e->all_dev, n_list, vars[s].vec, 0, 3);
-    return vars[s].supports(p) && vars[s].pays(p) ? s : vi;
+    return vars[s].supports(p) && ((e->variant_tuned && n_list == e->n) || vars[s].pays(p)) ? s : single;
 }
 
 int check_sticky(lbm_ensemble* e)
@@ -1145,7 +1145,7 @@ int lbm_ensemble_create(const lbm_config* cfg, int32_t n_clones, uint64_t seed, 
     e->clone_stride = 9 * e->plane;
     e->scale = (float)std::ldexp(1.0, c.storage == kFP32 ? 0 : c.shift_exp);
     e->inv_scale = (float)std::ldexp(1.0, c.storage == kFP32 ? 0 : -c.shift_exp);
-    e->variant = default_variant(c.storage);
+    e->variant = e->variant_single = default_variant(c.storage);
     e->perturb_mode = 0;
     e->variant_small = default_variant_small(c.storage, c.open_x != 0);
     e->use_graphs = true;
@@ -1633,8 +1633,9 @@ int lbm_ensemble_autotune(lbm_ensemble* e, int32_t* variant)
     LBM_CUDA(cudaEventCreate(&b));
     // Every trial launch reads the current buffer and rewrites the other one
     // at step_in_batch 0: the state does not advance and no drag is recorded.
-    auto tune = [&](int n_list, int reps, int best) -> int {
-        float best_ms = std::numeric_limits<float>::infinity();
+    // *single: the fastest but the row-streaming one, for the calls that do not stream
+    auto tune = [&](int n_list, int reps, int best, int* single) -> int {
+        float best_ms = std::numeric_limits<float>::infinity(), single_ms = best_ms;
         for (size_t i = 0; i < vars.size(); ++i) {
             const StepVariant& v = vars[i];
             if (v.storage != e->cfg.storage) continue;
@@ -1658,17 +1659,23 @@ int lbm_ensemble_autotune(lbm_ensemble* e, int32_t* variant)
                 best_ms = ms;
                 best = (int)i;
             }
+            if (v.kind != 3 && ms < single_ms) {
+                single_ms = ms;
+                *single = (int)i;
+            }
         }
         return best;
     };
     // the wide variant on the whole ensemble; the small-list one on a single
     // clone (one AMS branch), with more launches since each is short
-    const int wide = tune(e->n, 5, e->variant);
-    const int small = wide < 0 ? -1 : tune(1, 40, e->variant_small);
+    int single = default_variant(e->cfg.storage), unused = -1;
+    const int wide = tune(e->n, 5, e->variant, &single);
+    const int small = wide < 0 ? -1 : tune(1, 40, e->variant_small, &unused);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     if (wide < 0 || small < 0) return cuda_fail(cudaGetLastError(), "lbm_ensemble_autotune trial launch");
     e->variant = wide;
+    e->variant_single = single;
     e->variant_small = small;
     e->variant_tuned = true;
     e->variant_forced = false;

@@ -151,3 +151,34 @@ def test_default_streams_where_it_pays(L, n, nx, ny, storage, kw, streams):
     assert launches == (5 if streams else 9 + (1 if kw.get("open_x") else 0))
     ref = run(L, cfg, n, (8,), variant(L, storage, 0))
     assert np.array_equal(drag, ref[0]) and all(np.array_equal(x, y) for x, y in zip(pops, ref[1]))
+
+
+@pytest.mark.parametrize("n,nx,ny,storage,kw", [
+    (28, 512, 128, "fp32", dict(obstacle=(122, 56, 16, 16))),  # six rows a block
+    (152, 256, 64, "fp32", dict(obstacle=(50, 16, 32, 32))),   # streams faster, but not by default
+    (52, 512, 128, "fp16", dict(obstacle=(122, 56, 16, 16))),
+    (48, 512, 128, "fp32", dict(obstacle=(120, 56, 16, 16))),
+    (30, 1024, 256, "fp32", dict(obstacle=(158, 28, 200, 200))),
+])
+def test_tuned_variant_is_the_one_that_runs(L, n, nx, ny, storage, kw):
+    """eight steps take the launches of the variant that autotune returned; with three
+    steps, and while observables are recorded, a streaming choice makes way for single
+    steps, and the states do not depend on any of it"""
+    cfg = L.config(nx, ny, max_steps=32, storage=storage, tau=0.53, **kw)
+    ref = run(L, cfg, n, (8, 3, 4), variant(L, storage, 0))
+    e = L.lbm_ensemble_create(cfg, n, 5, torch.cuda.current_stream())
+    try:
+        kind = L.lbm_step_variant_kind(L.lbm_ensemble_autotune(e))
+        launches = []
+        for steps, observe in ((8, False), (3, False), (4, True)):
+            if observe:
+                L.lbm_ensemble_set_observables(e, True)
+            l0 = L.lbm_launch_count()
+            L.lbm_ensemble_step(e, steps)
+            launches.append(L.lbm_launch_count() - l0)
+        assert launches[0] == {0: 9, 1: 9, 2: 5, 3: 5}[kind], kind
+        assert launches[1] in (4, 2) and launches[2] == 4 + 4 + 1
+        for c, f in zip(sorted({0, n // 2, n - 1}), ref[1]):
+            assert np.array_equal(L.lbm_ensemble_get_populations(e, c, nx, ny), f)
+    finally:
+        L.lbm_ensemble_destroy(e)
