@@ -7,9 +7,10 @@
 //
 // Every result is the same bits as the scalar collision's: the packed forms
 // round each half as the scalar instructions do, and the fused multiply-adds
-// below are the ones the compiler forms from the scalar expressions (compared
-// over random states, with and without force, and over every FP32 argument of
-// the reciprocal from 5e-8 to 1e30).
+// below are the ones the compiler forms from the scalar expressions.  A compiler
+// that formed others would show where every variant of the step is run from one
+// random state far from equilibrium (tests/test_gpu_packed.py: both collisions,
+// periodic with force, open with varying rates, three storage formats).
 #pragma once
 #include "lbm_device.cuh"
 #include "step_params.h"
