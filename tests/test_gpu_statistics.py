@@ -114,3 +114,18 @@ def test_captured_autocorrelation_outlives_the_workspace(L):
         assert torch.equal(small, direct) and float(direct[0]) != 0.0
         assert torch.equal(large, before)
         del g
+
+
+@pytest.mark.parametrize("window,t_begin", [(1000, 0), (7, 3), (65, 69000)])
+def test_scores_of_a_series_longer_than_the_block_table(L, window, t_begin):
+    """trailing means of 70000 steps: the opening sums' blocks hold 35 steps there, 32
+    below 65537 (bounds as for the short series: 1e-11)"""
+    rng = np.random.default_rng(5)
+    d = 0.4 + np.cumsum(rng.normal(0, 1e-4, (2, 70000)), axis=1)
+    with Series(L, d) as e:
+        q = torch.zeros(2, dtype=torch.float64, device="cuda")
+        L.lbm_ensemble_scores(e, window, t_begin, 70000, q)
+        got = q.cpu().numpy()
+    s = np.concatenate([np.zeros((2, 1)), np.cumsum(d[:, t_begin:].astype(np.longdouble), axis=1)], axis=1)
+    ref = ((s[:, window:] - s[:, :-window]).max(axis=1) / window).astype(np.float64)
+    assert np.allclose(got, ref, rtol=1e-11, atol=1e-14)
