@@ -87,21 +87,18 @@ K_SIGMA = 1.0
 SIGMA_DRAG = 1e-3        # drag scale used to set k (k = K_SIGMA / (SIGMA_DRAG * PERIOD))
 BYTES_PER_SITE = 72      # FP32: 9 loads + 9 stores of 4 bytes
 METRIC = "Ensemble D2Q9 GLUPS & HBM-roofline fraction; time-to-return-time vs plain"
-# DRAM traffic of one fused-step launch measured by ncu (dram__bytes_read.sum +
-# dram__bytes_write.sum of launches of the full workload), per site,
+# DRAM traffic of a fused step measured by ncu (dram__bytes_read.sum +
+# dram__bytes_write.sum of launches of the full workload, over their steps), per site,
 # with the kernel sources it was measured on: reported only while they match
+STREAM_FILES = ("lbm_step_stream.cuh", "lbm_pair.cuh", "lbm_step.cuh", "lbm_device.cuh", "async_copy.cuh",
+                "step_params.h")
 NCU_TRAFFIC = {
-    ("gktl", "step_kernel<fp32, vec=4>"): {
-        "files": ("lbm_step.cuh", "lbm_device.cuh", "step_params.h", "step_fp32.cu"),
-        "sha": "241df406e4de695e", "bytes_per_site": 68.4597},
-    ("precision", "step_rows_kernel<fp16, vec=4>"): {
-        "files": ("lbm_step_rows.cuh", "async_copy.cuh", "lbm_step.cuh", "lbm_device.cuh", "step_params.h",
-                  "step_fp16.cu"),
-        "sha": "9c24a2e7bd8f6b3e", "bytes_per_site": 32.5115},
-    # both kernels of an open-channel step (the step kernel and the outlet kernel)
-    ("open", "step_kernel<fp32, vec=4, open> + open_bc_kernel"): {
-        "files": ("lbm_step.cuh", "lbm_device.cuh", "step_params.h", "step_open_fp32.cu"),
-        "sha": "3f91ba9496814b0e", "bytes_per_site": 59.1880},
+    ("gktl", "step_stream_kernel<fp32, vec=4>"): {
+        "files": STREAM_FILES + ("step_fp32.cu",), "sha": "51ffa3d984eb2b66", "bytes_per_site": 35.2292},
+    ("precision", "step_stream_kernel<fp16, vec=8>"): {
+        "files": STREAM_FILES + ("step_fp16.cu",), "sha": "bc0b1f18bd238614", "bytes_per_site": 16.7438},
+    ("open", "step_stream_kernel<fp32, vec=4, open> + open_bc_kernel"): {
+        "files": STREAM_FILES + ("step_open_fp32.cu",), "sha": "646a27f79b12693e", "bytes_per_site": 38.1242},
 }
 
 
@@ -111,7 +108,7 @@ def traffic_key(label: str) -> str:
     return re.sub(r", warps=\d+", "", label)
 
 
-def kernel_sha(files=NCU_TRAFFIC[("gktl", "step_kernel<fp32, vec=4>")]["files"]) -> str:
+def kernel_sha(files) -> str:
     h = hashlib.sha256()
     for f in files:
         with open(os.path.join(ROOT, "paper_2005_09323_gb300", "csrc", f), "rb") as fh:
